@@ -615,20 +615,27 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
     const int nblk = (n + kDiffNT - 1) / kDiffNT;
     const int nchunks = (a.D + kDC - 1) / kDC;
     const size_t part_pair = (size_t)nchunks * nblk * 4;
-    const size_t armc_n = armc_words(X, Y, a.wy);
     const float inv_tau = 1.f / a.tau;
     const dim3 tiles((X + kTileX - 1) / kTileX, (Y + kTileY - 1) / kTileY, B);
     static_assert(kTileX * kTileY == kDiffNT, "one thread per pixel of a tile");
     cudaError_t e = cudaSuccess;
     // frozen supports of every pair (integer path), support sizes, float grey
     diff_grey_kernel<<<dim3(nblk, 2, B), kDiffNT, 0, s>>>(a.left, a.right, w.gl, w.gr, n);
+    // (the arms of the left images only: nothing here uses the right base)
     for (int b = 0; b < B; ++b) {
         const size_t o = (size_t)b * n;
-        if ((e = launch_grey(a.left_u8 + o * 3, a.right_u8 + o * 3, w.ql + o, w.qr + o, X, Y, s)) != cudaSuccess ||
-            (e = launch_support(w.ql + o, w.qr + o, w.pixl + o, w.pixr + o, w.arml + o, w.armr + o,
-                                w.armcl + b * armc_n, w.armcr + b * armc_n, w.keyl + o, w.keyr + o, a.err, X, Y,
-                                a.wx, a.wy, a.tc, s)) != cudaSuccess)
+        if ((e = launch_grey(a.left_u8 + o * 3, a.right_u8 + o * 3, w.ql + o, w.qr + o, X, Y, s)) != cudaSuccess)
             return e;
+    }
+    for (int b0 = 0; b0 < B; b0 += kMaxSupImages / 2) {
+        SupImage im[kMaxSupImages];
+        const int nb = min(B - b0, kMaxSupImages / 2);
+        for (int k = 0; k < nb; ++k) {
+            const size_t o = (size_t)(b0 + k) * n;
+            im[2 * k] = SupImage{w.ql + o, w.pixl + o, w.arml + o, nullptr, nullptr, X, Y, 0};
+            im[2 * k + 1] = SupImage{w.qr + o, w.pixr + o, nullptr, nullptr, nullptr, X, Y, 0};
+        }
+        if ((e = launch_support(im, 2 * nb, a.wx, a.wy, a.tc, false, a.err, s)) != cudaSuccess) return e;
     }
     diff_nsupport_kernel<<<dim3(nblk, B), kDiffNT, 0, s>>>(w.arml, X, Y, w.ns);
     if (a.backward) {

@@ -26,6 +26,10 @@ __host__ __device__ inline size_t armc_index(int r, int x, int X)
 }
 inline size_t armc_words(int X, int Y, int wy) { return (size_t)X * (size_t)((Y + wy + 3) / 4) * 4; }
 
+// Ring slot of the vertical prefix before row i (64 slots), times two: as byte 1
+// of a word it is the byte offset of a 512-byte slot.
+__host__ __device__ inline uint32_t vslot(int i) { return (uint32_t)(i & 63) << 1; }
+
 // Tile shape of the fused kernel (see costagg.cu).
 constexpr int kRing = 64;      // V-prefix ring depth: 2*wy + 2 <= 64
 constexpr int kMaxWy = 31;
@@ -125,12 +129,20 @@ cudaError_t launch_grey_down(const uint8_t *rgb_l, const uint8_t *rgb_r, uint8_t
                             uint8_t *s_l, uint8_t *s_r, int W, int H, cudaStream_t s, int *launches);
 cudaError_t launch_downscale(const uint8_t *g_l, const uint8_t *g_r, uint8_t *s_l, uint8_t *s_r,
                              int W, int H, cudaStream_t s);
-// Also presets the WTA keys of both bases to ~0 and clears the fused
-// kernel's error word for this frame.
-cudaError_t launch_support(const uint8_t *g_l, const uint8_t *g_r, uint32_t *pix_l, uint32_t *pix_r,
-                           uint32_t *arm_l, uint32_t *arm_r, uint32_t *armc_l, uint32_t *armc_r,
-                           uint32_t *key_l, uint32_t *key_r, uint32_t *err, int X, int Y, int wx, int wy,
-                           int tc, cudaStream_t s);
+// Mini-census codes and cross arms of up to kMaxSupImages images in one launch
+// (nx is filled by the launcher). Also presets the WTA keys to ~0 where key is
+// given, and clears the fused kernel's error word. wide: armc takes the
+// vertical slots of the two-pass kernel (vslot), else the fused kernel's rows
+// (armc_index).
+constexpr int kMaxSupImages = 64;
+struct SupImage {
+    const uint8_t *g;                  // grey [Y][X]
+    uint32_t *pix;                     // [Y][X]
+    uint32_t *arm, *armc, *key;        // may be null: not wanted (armc and key need arm)
+    int X, Y, nx;                      // size, tiles per row
+};
+cudaError_t launch_support(const SupImage *im, int n, int wx, int wy, int tc, bool wide, uint32_t *err,
+                           cudaStream_t s);
 cudaError_t launch_costagg(const CostAggArgs &a, cudaStream_t s);
 cudaError_t launch_refine(const uint32_t *key_l, const uint32_t *key_r, const uint8_t *grey_l,
                           int X, int Y, int T, int fill_mode, uint8_t *dl, uint8_t *dr, uint8_t *gcp,

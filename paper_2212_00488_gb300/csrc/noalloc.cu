@@ -124,9 +124,12 @@ extern "C" int stereo_compute_noalloc(const stereo_params *params, const uint8_t
     if ((e = ds ? launch_grey_down(left_rgb, right_rgb, u8(o_gf[0]), u8(o_gf[1]), u8(o_gs[0]), u8(o_gs[1]), W, H,
                                    s, &launches)
                 : launch_grey(left_rgb, right_rgb, u8(o_gf[0]), u8(o_gf[1]), W, H, s)) == cudaSuccess &&
-        (e = launch_support(u8(o_gs[0]), u8(o_gs[1]), u32(o_pix[0]), u32(o_pix[1]), u32(o_arm[0]), u32(o_arm[1]),
-                            u32(o_armc[0]), u32(o_armc[1]), u32(o_key[0]), u32(o_key[1]), u32(o_err), X, Y, p.wx,
-                            p.wy, p.tc, s)) == cudaSuccess) {
+        (e = [&] {
+            SupImage im[2];
+            for (int i = 0; i < 2; ++i)
+                im[i] = SupImage{u8(o_gs[i]), u32(o_pix[i]), u32(o_arm[i]), u32(o_armc[i]), u32(o_key[i]), X, Y, 0};
+            return launch_support(im, 2, p.wx, p.wy, p.tc, false, u32(o_err), s);
+        }()) == cudaSuccess) {
         CostAggArgs a{};
         a.pix_l = u32(o_pix[0]);
         a.pix_r = u32(o_pix[1]);

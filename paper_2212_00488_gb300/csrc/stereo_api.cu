@@ -252,9 +252,12 @@ cudaError_t run_stage(stereo_ctx *c, int stage, cudaStream_t s)
     }
     case STEREO_STAGE_SUPPORT:
         c->launches++;
-        return launch_support(c->gs[0], c->gs[1], c->pix[0], c->pix[1], c->arm[0], c->arm[1], c->armc[0],
-                              c->armc[1], c->key[0], c->key[1], c->d_err, c->X, c->Y, c->p.wx, c->p.wy,
-                              c->p.tc, s);
+        {
+            SupImage im[2];
+            for (int i = 0; i < 2; ++i)
+                im[i] = SupImage{c->gs[i], c->pix[i], c->arm[i], c->armc[i], c->key[i], c->X, c->Y, 0};
+            return launch_support(im, 2, c->p.wx, c->p.wy, c->p.tc, false, c->d_err, s);
+        }
     case STEREO_STAGE_COSTAGG: {
         CostAggArgs a;
         a.pix_l = c->pix[0];
@@ -689,18 +692,28 @@ CostAggArgs frame_args(const stereo_ctx *c, const FrameWs &f)
     return a;
 }
 
-cudaError_t batch_prep(stereo_ctx *c, const stereo_job &j, const FrameWs &f, cudaStream_t s, int &launches)
+// Grey, downscale and supports of every frame of a batch: one support launch
+// for all of them.
+cudaError_t batch_prep(stereo_ctx *c, const std::vector<const stereo_job *> &jobs, const std::vector<FrameWs> &fw,
+                       cudaStream_t s, int &launches)
 {
-    cudaError_t e;
-    if (c->p.downscale) {
-        e = launch_grey_down(j.left_rgb, j.right_rgb, f.gf[0], f.gf[1], f.gs[0], f.gs[1], f.W, f.H, s, &launches);
-    } else {
-        e = launch_grey(j.left_rgb, j.right_rgb, f.gf[0], f.gf[1], f.W, f.H, s);
-        launches++;
+    cudaError_t e = cudaSuccess;
+    SupImage im[2 * kMaxBatch];
+    const int n = (int)fw.size();
+    for (int k = 0; k < n && e == cudaSuccess; ++k) {
+        const stereo_job &j = *jobs[k];
+        const FrameWs &f = fw[k];
+        if (c->p.downscale) {
+            e = launch_grey_down(j.left_rgb, j.right_rgb, f.gf[0], f.gf[1], f.gs[0], f.gs[1], f.W, f.H, s, &launches);
+        } else {
+            e = launch_grey(j.left_rgb, j.right_rgb, f.gf[0], f.gf[1], f.W, f.H, s);
+            launches++;
+        }
+        for (int i = 0; i < 2; ++i)
+            im[2 * k + i] = SupImage{f.gs[i], f.pix[i], f.arm[i], f.armc[i], f.key[i], f.X, f.Y, 0};
     }
     if (e == cudaSuccess) {
-        e = launch_support(f.gs[0], f.gs[1], f.pix[0], f.pix[1], f.arm[0], f.arm[1], f.armc[0], f.armc[1],
-                           f.key[0], f.key[1], c->d_err, f.X, f.Y, c->p.wx, c->p.wy, c->p.tc, s);
+        e = launch_support(im, 2 * n, c->p.wx, c->p.wy, c->p.tc, false, c->d_err, s);
         launches++;
     }
     return e;
@@ -787,11 +800,13 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
         c->bws_size = need;
     }
     std::vector<FrameWs> fw(n);
+    std::vector<const stereo_job *> ordered(n);
     BatchArgs b{};
     b.njobs = n;
     b.counter = (uint32_t *)c->bws;
     for (int k = 0; k < n; ++k) {
         const stereo_job &j = jobs[order[k]];
+        ordered[k] = &j;
         frame_layout(c->p, j.W, j.H, j.Dmax, (char *)c->bws + offs[k], &fw[k]);
         b.job[k] = frame_args(c, fw[k]);
     }
@@ -817,9 +832,7 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
         } else {
             // the autotuner: run the preparation once, then time each tile
             // shape that fits every job (one warm-up and two timed launches)
-            for (int k = 0; k < n; ++k)
-                if ((e = batch_prep(c, jobs[order[k]], fw[k], s, launches)) != cudaSuccess)
-                    return cuda_fail(c, e, "kernel launch");
+            if ((e = batch_prep(c, ordered, fw, s, launches)) != cudaSuccess) return cuda_fail(c, e, "kernel launch");
             float best = 0.f;
             for (int t = 0; t < kNumTiles; ++t) {
                 c->last_batch_tune_ms[t] = -1.f;
@@ -853,7 +866,7 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
     launches = 0;
     if ((e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
         return cuda_fail(c, e, "stream capture");
-    for (int k = 0; k < n && e == cudaSuccess; ++k) e = batch_prep(c, jobs[order[k]], fw[k], s, launches);
+    e = batch_prep(c, ordered, fw, s, launches);
     if (e == cudaSuccess) {
         e = launch_costagg_batch(b, tile, c->num_sms, s);
         launches++;
