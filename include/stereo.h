@@ -193,13 +193,14 @@ STEREO_API int stereo_last_launch_count(const stereo_ctx *ctx);
 /* Tile shapes of the fused cost + aggregation + WTA kernel (columns per base
  * x disparities per CTA, row-prefix width); every consumer thread holds one
  * column and 4 disparities of its tile:
- * 0: 104x4 16-bit for wx up to 26, 1: 104x4 16-bit for wx up to 58,
- * 2: 104x4 32-bit for wx up to 26, 3: 104x4 32-bit for wx up to 58,
- * 4: 64x4 16-bit, 5: 100x4 16-bit with 12 row-prefix producer warps
- * instead of 8, 6: 48x8 32-bit (slabs of 8 disparities, two threads per
- * column), 7: 64x4 32-bit for wx up to 174 with 8 producer warps (the wide
+ * 0: 96x4 16-bit for wx up to 26 with 12 row-prefix producer warps, 1: 96x4
+ * 16-bit for wx up to 58, 2: 104x4 32-bit for wx up to 26, 3: 104x4 32-bit for
+ * wx up to 58, 4: 64x4 16-bit for wx up to 46 with 16 producer warps, 5: 100x4
+ * 16-bit for wx up to 28, 6: 48x8 32-bit (slabs of 8 disparities, two threads
+ * per column), 7: 64x4 32-bit for wx up to 174 with 8 producer warps (the wide
  * windows of Table I, up to the library's limit of 141), 8: 88x4 32-bit for
- * wx up to 66 with 8 producer warps.
+ * wx up to 66 with 8 producer warps. A frame whose tiles leave SMs idle is cut
+ * into bands of rows, each with its own tiles.
  * 16-bit row prefixes need max(2*wx+1, 7) times the largest matching cost
  * below 2^16. Every shape gives the same result; they differ only in speed.
  * A compute with a shape that does not fit the parameters fails with EINVAL. */

@@ -635,7 +635,7 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
             im[2 * k] = SupImage{w.ql + o, w.pixl + o, w.arml + o, nullptr, nullptr, X, Y, 0};
             im[2 * k + 1] = SupImage{w.qr + o, w.pixr + o, nullptr, nullptr, nullptr, X, Y, 0};
         }
-        if ((e = launch_support(im, 2 * nb, a.wx, a.wy, a.tc, false, a.err, s)) != cudaSuccess) return e;
+        if ((e = launch_support(im, 2 * nb, a.wx, a.wy, a.tc, a.err, s)) != cudaSuccess) return e;
     }
     diff_nsupport_kernel<<<dim3(nblk, B), kDiffNT, 0, s>>>(w.arml, X, Y, w.ns);
     if (a.backward) {

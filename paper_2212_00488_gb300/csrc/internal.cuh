@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 namespace stereo {
 
 // Packed per-pixel words written by the support stage and read by the fused
@@ -18,17 +20,21 @@ __host__ __device__ inline uint32_t pack_arm(int hm, int hp, int vm, int vp)
 // Arm words of the fused kernel, row quads interleaved: the word of row r and
 // column x sits at ((r / 4) X + x) 4 + r % 4, so one 16-byte load fetches a
 // column's words of four consecutive rows. Row r holds the left/right arms of
-// row r (low half) and the up/down arms of row r - wy (high half); rows run
-// to Y + wy - 1, rounded up to whole quads.
+// row r (low half) and the ring slots of the vertical window of row r - wy
+// (high half, armc_slots; 0 where there is no such row); rows run to Y + wy - 1,
+// rounded up to whole quads.
 __host__ __device__ inline size_t armc_index(int r, int x, int X)
 {
     return ((size_t)(r >> 2) * X + x) * 4 + (r & 3);
 }
+// Ring slots of the vertical prefixes at both ends of the window of row y with
+// arms up and down: V(y - up) in the low byte, V(y + down + 1) in the high one
+// (the prefix before row r sits in slot (r - 1) mod 64).
+__host__ __device__ inline uint32_t armc_slots(int y, int up, int down)
+{
+    return (uint32_t)((y - up - 1) & 63) | (uint32_t)((y + down) & 63) << 8;
+}
 inline size_t armc_words(int X, int Y, int wy) { return (size_t)X * (size_t)((Y + wy + 3) / 4) * 4; }
-
-// Ring slot of the vertical prefix before row i (64 slots), times two: as byte 1
-// of a word it is the byte offset of a 512-byte slot.
-__host__ __device__ inline uint32_t vslot(int i) { return (uint32_t)(i & 63) << 1; }
 
 // Tile shape of the fused kernel (see costagg.cu).
 constexpr int kRing = 64;      // V-prefix ring depth: 2*wy + 2 <= 64
@@ -49,6 +55,7 @@ struct CostAggArgs {
     uint32_t P;                      // cost of a match outside the image
     int tile;                        // tile shape id, -1 = pick from the shape
     int num_sms;                     // SMs of the device (for the pick)
+    int band;                        // rows of a band (filled by the launcher)
 };
 
 // Programmatic dependent launch between the kernels of a frame: a kernel
@@ -131,9 +138,7 @@ cudaError_t launch_downscale(const uint8_t *g_l, const uint8_t *g_r, uint8_t *s_
                              int W, int H, cudaStream_t s);
 // Mini-census codes and cross arms of up to kMaxSupImages images in one launch
 // (nx is filled by the launcher). Also presets the WTA keys to ~0 where key is
-// given, and clears the fused kernel's error word. wide: armc takes the
-// vertical slots of the two-pass kernel (vslot), else the fused kernel's rows
-// (armc_index).
+// given, and clears the fused kernel's error word.
 constexpr int kMaxSupImages = 64;
 struct SupImage {
     const uint8_t *g;                  // grey [Y][X]
@@ -141,8 +146,7 @@ struct SupImage {
     uint32_t *arm, *armc, *key;        // may be null: not wanted (armc and key need arm)
     int X, Y, nx;                      // size, tiles per row
 };
-cudaError_t launch_support(const SupImage *im, int n, int wx, int wy, int tc, bool wide, uint32_t *err,
-                           cudaStream_t s);
+cudaError_t launch_support(const SupImage *im, int n, int wx, int wy, int tc, uint32_t *err, cudaStream_t s);
 cudaError_t launch_costagg(const CostAggArgs &a, cudaStream_t s);
 cudaError_t launch_refine(const uint32_t *key_l, const uint32_t *key_r, const uint8_t *grey_l,
                           int X, int Y, int T, int fill_mode, uint8_t *dl, uint8_t *dr, uint8_t *gcp,

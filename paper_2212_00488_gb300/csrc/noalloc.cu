@@ -128,7 +128,7 @@ extern "C" int stereo_compute_noalloc(const stereo_params *params, const uint8_t
             SupImage im[2];
             for (int i = 0; i < 2; ++i)
                 im[i] = SupImage{u8(o_gs[i]), u32(o_pix[i]), u32(o_arm[i]), u32(o_armc[i]), u32(o_key[i]), X, Y, 0};
-            return launch_support(im, 2, p.wx, p.wy, p.tc, false, u32(o_err), s);
+            return launch_support(im, 2, p.wx, p.wy, p.tc, u32(o_err), s);
         }()) == cudaSuccess) {
         CostAggArgs a{};
         a.pix_l = u32(o_pix[0]);

@@ -273,7 +273,6 @@ __device__ __forceinline__ void scan_y(const uint32_t *col, int cap, uint32_t bm
 template <int N>
 struct SupArgs {
     int n, wx, wy, tc;
-    int wide;                                // armc holds the vertical slots of the two-pass kernel, not its own layout
     uint32_t *err;
     int start[N + 1];                        // first CTA of each image
     SupImage im[N];
@@ -347,7 +346,6 @@ __global__ void __launch_bounds__(kSupNT, 3) support_kernel(const __grid_constan
     if (x >= X) return;
     const uint8_t *rb = reinterpret_cast<const uint8_t *>(res) + 4 * q * kSX + ox;
     const uint8_t *gb = reinterpret_cast<const uint8_t *>(rows + (1 + 4 * q) * RW + hw) + ox;
-    uint32_t slots[2] = {0u, 0u};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int y = y0 + 4 * q + j;
@@ -361,17 +359,17 @@ __global__ void __launch_bounds__(kSupNT, 3) support_kernel(const __grid_constan
         const int u = min((int)rb[(2 * kSY + j) * kSX], y), d = min((int)rb[(3 * kSY + j) * kSX], Y - 1 - y);
         I.arm[i] = pack_arm(l, r, u, d);
         if (!I.armc) continue;
-        if (A.wide) {
-            slots[j >> 1] |= (vslot(y - u) | vslot(y + d + 1) << 8) << (16 * (j & 1));
-        } else {
-            uint16_t *ac = reinterpret_cast<uint16_t *>(I.armc);
-            ac[2 * armc_index(y, x, X)] = (uint16_t)(l | r << 8);
-            // the fused kernel reads the up/down arms of output row y in row y + wy
-            ac[2 * armc_index(y + wy, x, X) + 1] = (uint16_t)(u | d << 8);
+        uint16_t *ac = reinterpret_cast<uint16_t *>(I.armc);
+        ac[2 * armc_index(y, x, X)] = (uint16_t)(l | r << 8);
+        // the fused kernel takes output row y in row y + wy; it reads the rows
+        // before and after those too, and does nothing with them
+        ac[2 * armc_index(y + wy, x, X) + 1] = (uint16_t)armc_slots(y, u, d);
+        if (y < wy) ac[2 * armc_index(y, x, X) + 1] = 0;
+        if (y == Y - 1) {
+            for (int i = Y; i < wy; ++i) ac[2 * armc_index(i, x, X) + 1] = 0;
+            for (int i = Y + wy; i & 3; ++i) ac[2 * armc_index(i, x, X) + 1] = 0;
         }
     }
-    if (I.arm && I.armc && A.wide && y0 + 4 * q < Y)
-        reinterpret_cast<uint2 *>(I.armc)[(size_t)(y0 / 4 + q) * X + x] = make_uint2(slots[0], slots[1]);
 }
 
 __global__ void unpack_kernel(const uint32_t *__restrict__ pix, const uint32_t *__restrict__ arm,
@@ -434,14 +432,13 @@ cudaError_t launch_grey_down(const uint8_t *rgb_l, const uint8_t *rgb_r, uint8_t
 namespace {
 
 template <int N>
-cudaError_t support_run(const SupImage *im, int n, int wx, int wy, int tc, bool wide, uint32_t *err, cudaStream_t s)
+cudaError_t support_run(const SupImage *im, int n, int wx, int wy, int tc, uint32_t *err, cudaStream_t s)
 {
     SupArgs<N> A;
     A.n = n;
     A.wx = wx;
     A.wy = wy;
     A.tc = tc;
-    A.wide = wide;
     A.err = err;
     A.start[0] = 0;
     for (int i = 0; i < n; ++i) {
@@ -456,13 +453,12 @@ cudaError_t support_run(const SupImage *im, int n, int wx, int wy, int tc, bool 
 
 }  // namespace
 
-cudaError_t launch_support(const SupImage *im, int n, int wx, int wy, int tc, bool wide, uint32_t *err,
-                           cudaStream_t s)
+cudaError_t launch_support(const SupImage *im, int n, int wx, int wy, int tc, uint32_t *err, cudaStream_t s)
 {
     if (n < 1 || n > kMaxSupImages || wx > kMaxWx || wy > kMaxWy) return cudaErrorInvalidValue;
     // the kernel's argument holds every image: two for a frame, more for a batch
-    return n <= 2 ? support_run<2>(im, n, wx, wy, tc, wide, err, s)
-                  : support_run<kMaxSupImages>(im, n, wx, wy, tc, wide, err, s);
+    return n <= 2 ? support_run<2>(im, n, wx, wy, tc, err, s)
+                  : support_run<kMaxSupImages>(im, n, wx, wy, tc, err, s);
 }
 
 cudaError_t launch_unpack_planes(const uint32_t *pix, const uint32_t *arm, uint8_t *grey,

@@ -256,7 +256,7 @@ cudaError_t run_stage(stereo_ctx *c, int stage, cudaStream_t s)
             SupImage im[2];
             for (int i = 0; i < 2; ++i)
                 im[i] = SupImage{c->gs[i], c->pix[i], c->arm[i], c->armc[i], c->key[i], c->X, c->Y, 0};
-            return launch_support(im, 2, c->p.wx, c->p.wy, c->p.tc, false, c->d_err, s);
+            return launch_support(im, 2, c->p.wx, c->p.wy, c->p.tc, c->d_err, s);
         }
     case STEREO_STAGE_COSTAGG: {
         CostAggArgs a;
@@ -713,7 +713,7 @@ cudaError_t batch_prep(stereo_ctx *c, const std::vector<const stereo_job *> &job
             im[2 * k + i] = SupImage{f.gs[i], f.pix[i], f.arm[i], f.armc[i], f.key[i], f.X, f.Y, 0};
     }
     if (e == cudaSuccess) {
-        e = launch_support(im, 2 * n, c->p.wx, c->p.wy, c->p.tc, false, c->d_err, s);
+        e = launch_support(im, 2 * n, c->p.wx, c->p.wy, c->p.tc, c->d_err, s);
         launches++;
     }
     return e;

@@ -1,0 +1,42 @@
+"""Row bands and slab edges of the fused kernel against the oracle, integer for
+integer: frames tall and narrow enough to be cut into bands, arms at the caps so
+that windows cross every band border, strips one column either side of a tile's
+width, and disparity counts that make the last slab overlap the one before it
+(or fall short of one slab)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2212_00488_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2212_00488_gb300 import build
+    build.build()
+
+
+@pytest.mark.parametrize("tile", [-1, 0, 3, 4, 5, 8])
+@pytest.mark.parametrize("W,H,D", [(40, 901, 9), (95, 130, 3), (96, 61, 4), (97, 300, 5), (193, 257, 75)])
+def test_bands_and_overlapping_slabs(W, H, D, tile):
+    from paper_2212_00488_gb300 import Stereo, _lib
+    s = scenes.make_scene(W, H, D, planes=5, seed=W + H)
+    left, right = s.left // 64 + 100, s.right // 64 + 100          # arms at their caps
+    st = Stereo(0, downscale=0)
+    _lib.stereo_set_tile(st.ctx, tile)
+    out = st(torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda(), D, maps=True)
+    torch.cuda.synchronize()
+    st.close()
+    p = oracle.Params()
+    p.downscale = 0
+    ref = oracle.pipeline(left, right, D, p)
+    for k in ("dl", "dr", "gcp", "disp"):
+        got, want = getattr(out, k).cpu().numpy(), getattr(ref, k)
+        bad = np.argwhere(got != want)
+        assert bad.size == 0, f"{k}: {len(bad)} mismatches, first {bad[:5].tolist()}"
