@@ -13,13 +13,22 @@
 //
 // The volume is never stored: forward and backward walk the disparities in
 // chunks of kDC, keeping per chunk the x-aggregated slab and, in backward,
-// the slab's gradients. Every pair of the batch has its own buffers, and the
-// per-chunk kernels take all pairs in one launch (blockIdx.y = pair), so a
-// launch is several waves of blocks rather than one and a partial one. Sums
-// over arms are direct (at most 2 wx + 1 and 2 wy + 1 terms), which keeps FP32
-// aggregates within about 6e-6 of their exact value. The adjoint of each sum
-// is a banded difference array walked in a fixed order by one thread, so no
-// float atomics are used and results are deterministic.
+// the slab's gradients, all as [y][x][kDC] so that a pixel's disparities are two
+// 16-byte accesses. Every pair of the batch has its own buffers, and the
+// per-chunk kernels take all pairs in one launch.
+//
+// Sums over arms run over whole blocks of four cells where the window holds
+// them and single cells at its ends (step4), at most 3 + 10 + 3 terms along x
+// and 3 + 15 + 3 along y for the default caps: every term is a sum of cells of
+// the window itself, so an aggregate keeps the accuracy of a direct sum and a
+// NaN stays in the windows that hold it. The adjoint of each sum is a banded
+// difference array walked in a fixed order by one thread, so no float atomics
+// are used and results are deterministic.
+//
+// 4 pairs of 718 x 496, D 73, forward and backward (arms at their caps in a third
+// of the planes): 9.1 ms with direct sums over planes [kDC][y][x] and separate
+// kernels for the horizontal adjoint and the cost gradient, 4.2 ms now. Bound by
+// the L1 traffic of the vertical sums and the dependent chains of the adjoints.
 #include "internal.cuh"
 
 namespace stereo {
@@ -75,99 +84,160 @@ struct Theta {
 
 __device__ __forceinline__ Theta load_theta(const float *t) { return Theta{t[0], t[1], t[2], t[3]}; }
 
-// One block per row y and chunk: the cost rows of all disparities of the
-// chunk in shared memory ([dc][X]), then each pixel's own x window summed
-// directly, every plane in ascending x.
-__global__ void diff_costx_kernel(const float *__restrict__ gL, const float *__restrict__ gR,
-                                  const uint32_t *__restrict__ pixL, const uint32_t *__restrict__ pixR,
-                                  const uint32_t *__restrict__ arm, const float *__restrict__ theta, int X, int Y,
-                                  int D, int d0, int dc, float *__restrict__ cax)
+__device__ __forceinline__ void add4(float (&s)[kDC], int j, const float4 v)
 {
-    extern __shared__ float crow[];
-    const int y = blockIdx.x;
-    const size_t b = blockIdx.y, n = (size_t)X * Y;   // pair
+    s[j] += v.x;
+    s[j + 1] += v.y;
+    s[j + 2] += v.z;
+    s[j + 3] += v.w;
+}
+
+// The next term of a window sum over [t, hi]: a whole aligned block of four cells
+// if the window holds it, else cell t.
+__device__ __forceinline__ bool step4(int t, int hi) { return (t & 3) == 0 && t + 3 <= hi; }
+
+// Cost and x window sums. A block takes kCXSeg columns of a row quad: the costs
+// of the chunk's disparities for those columns and a wx halo go to shared memory
+// (two float4 planes per row), with the sums of aligned column quads beside
+// them; then a thread owns one column and sums its own windows. It also writes
+// the sum of its four rows, the blocks of the vertical sums.
+constexpr int kCXSeg = 256;
+static_assert(kCXSeg == kDiffNT, "one column per thread");
+
+__host__ __device__ __forceinline__ int costx_pitch(int X, int wx)
+{
+    return ((X < kCXSeg + 2 * wx + 4 ? X : kCXSeg + 2 * wx + 4) + 3) / 4 * 4;
+}
+size_t diff_costx_smem(int X, int wx) { return (size_t)costx_pitch(X, wx) * 5 / 4 * 4 * 2 * sizeof(float4); }
+
+__global__ void __launch_bounds__(kDiffNT) diff_costx_kernel(
+    const float *__restrict__ gL, const float *__restrict__ gR, const uint32_t *__restrict__ pixL,
+    const uint32_t *__restrict__ pixR, const uint32_t *__restrict__ arm, const float *__restrict__ theta, int X, int Y,
+    int D, int d0, int wx, float4 *__restrict__ hs, float4 *__restrict__ bs)
+{
+    extern __shared__ float4 csm[];
+    __shared__ float mc[8];
+    pdl_trigger();
+    const int x0 = blockIdx.x * kCXSeg, y0 = blockIdx.y * 4;
+    const size_t b = blockIdx.z, n = (size_t)X * Y;   // pair
+    const int P = costx_pitch(X, wx);
+    float4 *cell = csm, *quad = csm + 8 * P;          // [4 rows][2][P], [4 rows][2][P / 4]
+    pdl_wait();
     gL += b * n;
     gR += b * n;
     pixL += b * n;
     pixR += b * n;
     arm += b * n;
-    cax += b * kDC * n;
+    hs += b * 2 * n;
+    bs += b * 2 * X * (size_t)((Y + 3) / 4);
     const Theta th = load_theta(theta);
-    const float P = th.wad * (1.f - expf(-1.f / th.lad)) + th.wmc * (1.f - expf(-6.f / th.lmc));
-    const size_t r = (size_t)y * X;
-    const int kn = min(dc, D - d0);
+    const float Pc = th.wad * (1.f - expf(-1.f / th.lad)) + th.wmc * (1.f - expf(-6.f / th.lmc));
+    const int kn = min(kDC, D - d0);
     // the census term takes seven values: one exp per Hamming distance
-    __shared__ float mc[8];
     if (threadIdx.x < 7) mc[threadIdx.x] = th.wmc * (1.f - expf(-(float)threadIdx.x / th.lmc));
     const float inv_lad = 1.f / th.lad;
+    const int xs = max(x0 - wx, 0) & ~3, xe = min(x0 + kCXSeg + wx, X);   // staged columns
     __syncthreads();
-    for (int x = threadIdx.x; x < X; x += blockDim.x) {
-        const float gl = gL[r + x];
-        const uint32_t pl = pixL[r + x];
-        // the chunk's disparities unrolled, so their loads and exps overlap
+    for (int r = 0; r < 4 && y0 + r < Y; ++r) {
+        const size_t row = (size_t)(y0 + r) * X;
+        for (int x = xs + (int)threadIdx.x; x < xe; x += kDiffNT) {
+            const float gl = gL[row + x];
+            const uint32_t pl = pixL[row + x];
+            float c[kDC];
+            // the chunk's disparities unrolled, so their loads and exps overlap
 #pragma unroll
-        for (int k = 0; k < kDC; ++k) {
-            if (k < kn) {
+            for (int k = 0; k < kDC; ++k) {
                 const int d = d0 + k;
-                float c = P;
-                if (x >= d) {
-                    const float a = fabsf(gl - gR[r + x - d]);
-                    const int h = __popc((pl ^ pixR[r + x - d]) & 0x3F00u);
-                    c = th.wad * (1.f - expf(-a * inv_lad)) + mc[h];
+                c[k] = k < kn ? Pc : 0.f;
+                if (k < kn && x >= d) {
+                    const float a = fabsf(gl - gR[row + x - d]);
+                    const int h = __popc((pl ^ pixR[row + x - d]) & 0x3F00u);
+                    c[k] = th.wad * (1.f - expf(-a * inv_lad)) + mc[h];
                 }
-                crow[k * X + x] = c;
             }
+            cell[(2 * r) * P + x - xs] = make_float4(c[0], c[1], c[2], c[3]);
+            cell[(2 * r + 1) * P + x - xs] = make_float4(c[4], c[5], c[6], c[7]);
         }
     }
     __syncthreads();
-    for (int x = threadIdx.x; x < X; x += blockDim.x) {
-        const uint32_t am = arm[r + x];
-        const int lo = x - (int)(am & 0xFF), hi = x + (int)((am >> 8) & 0xFF);
+    const int nq = (xe - xs) / 4;                     // whole quads
+    for (int i = threadIdx.x; i < 8 * nq; i += kDiffNT) {
+        const int j = i / nq, q = i - j * nq;
+        if (y0 + j / 2 >= Y) break;
+        const float4 *c = cell + j * P + 4 * q;
+        const float4 u = c[0], v = c[1], w = c[2], z = c[3];
+        quad[j * (P / 4) + q] = make_float4(u.x + v.x + w.x + z.x, u.y + v.y + w.y + z.y, u.z + v.z + w.z + z.z,
+                                            u.w + v.w + w.w + z.w);
+    }
+    __syncthreads();
+    const int x = x0 + threadIdx.x;
+    if (x >= X) return;
+    float sum[kDC];
+#pragma unroll
+    for (int k = 0; k < kDC; ++k) sum[k] = 0.f;
+    for (int r = 0; r < 4 && y0 + r < Y; ++r) {
+        const size_t i = (size_t)(y0 + r) * X + x;
+        const uint32_t am = arm[i];
+        const int hi = x + (int)((am >> 8) & 0xFF) - xs;
+        const float4 *c0 = cell + 2 * r * P, *q0 = quad + 2 * r * (P / 4);
         float s[kDC];
 #pragma unroll
         for (int k = 0; k < kDC; ++k) s[k] = 0.f;
-        for (int t = lo; t <= hi; ++t) {
-#pragma unroll
-            for (int k = 0; k < kDC; ++k)
-                if (k < kn) s[k] += crow[k * X + t];
+        for (int t = x - (int)(am & 0xFF) - xs; t <= hi;) {
+            const bool four = step4(t, hi);
+            const float4 *p = four ? q0 + (t >> 2) : c0 + t;
+            add4(s, 0, p[0]);
+            add4(s, 4, p[four ? P / 4 : P]);
+            t += four ? 4 : 1;
         }
+        hs[2 * i] = make_float4(s[0], s[1], s[2], s[3]);
+        hs[2 * i + 1] = make_float4(s[4], s[5], s[6], s[7]);
 #pragma unroll
-        for (int k = 0; k < kDC; ++k)
-            if (k < kn) cax[((size_t)k * Y + y) * X + x] = s[k];
+        for (int k = 0; k < kDC; ++k) sum[k] += s[k];
     }
+    float4 *o = bs + 2 * ((size_t)(y0 / 4) * X + x);
+    o[0] = make_float4(sum[0], sum[1], sum[2], sum[3]);
+    o[1] = make_float4(sum[4], sum[5], sum[6], sum[7]);
 }
 
-// Vertical sums of Eq. 8 for the chunk's dc planes at once: one pass over the
-// anchor's span [y - up, y + down], each plane summed in ascending y.
-__device__ __forceinline__ void vsum_chunk(const float *__restrict__ cax, const uint32_t am, int x, int y, int X,
-                                           size_t plane, int dc, float (&out)[kDC])
+// Vertical sums of Eq. 8 for the chunk's disparities at once, over the anchor's
+// span [y - up, y + down]: row sums at its ends, the sums of whole row quads
+// between.
+__device__ __forceinline__ void vsum_chunk(const float4 *__restrict__ hs, const float4 *__restrict__ bs,
+                                           const uint32_t am, int x, int y, int X, float (&out)[kDC])
 {
-    const int up = (am >> 16) & 0xFF, down = am >> 24;
 #pragma unroll
     for (int k = 0; k < kDC; ++k) out[k] = 0.f;
-    for (int t = -up; t <= down; ++t) {
-        const float *p = cax + (size_t)(y + t) * X + x;
-#pragma unroll
-        for (int k = 0; k < kDC; ++k)
-            if (k < dc) out[k] += p[k * plane];
+    const int hi = y + (int)(am >> 24);
+    hs += 2 * x;
+    bs += 2 * x;
+    for (int t = y - (int)((am >> 16) & 0xFF); t <= hi;) {
+        const bool four = step4(t, hi);
+        const float4 *p = (four ? bs : hs) + (size_t)(four ? t >> 2 : t) * (2 * X);
+        add4(out, 0, p[0]);
+        add4(out, 4, p[1]);
+        t += four ? 4 : 1;
     }
 }
 
 // Forward: aggregated cost along y per pixel and an online softmax over d.
 // state = (max z, sum exp(z - max), sum d exp(z - max)) per pixel.
-__global__ void diff_vagg_softmax_kernel(const float *__restrict__ cax, const uint32_t *__restrict__ arm,
-                                         const float *__restrict__ ns, int X, int Y, int D, int d0, int dc,
-                                         float inv_tau, float *__restrict__ state, int first, int last,
+__global__ void diff_vagg_softmax_kernel(const float4 *__restrict__ hs, const float4 *__restrict__ bs,
+                                         const uint32_t *__restrict__ arm, const float *__restrict__ ns, int X, int Y,
+                                         int D, int d0, float inv_tau, float *__restrict__ state, int first, int last,
                                          float *__restrict__ dhat, float *__restrict__ stats)
 {
+    pdl_trigger();
     // 2-D tiles of kTileX x kTileY pixels: the warps of a block walk the
     // same anchor rows, so their vertical windows meet in L1
     const int x = blockIdx.x * kTileX + (int)(threadIdx.x % kTileX);
     const int y = blockIdx.y * kTileY + (int)(threadIdx.x / kTileX);
+    pdl_wait();
     if (x >= X || y >= Y) return;
     const int i = y * X + x;
     const size_t b = blockIdx.z, n = (size_t)X * Y;   // pair
-    cax += b * kDC * n;
+    hs += b * 2 * n;
+    bs += b * 2 * X * (size_t)((Y + 3) / 4);
     arm += b * n;
     ns += b * n;
     state += b * 3 * n;
@@ -178,10 +248,10 @@ __global__ void diff_vagg_softmax_kernel(const float *__restrict__ cax, const ui
     float m = first ? -INFINITY : state[3 * i], s = first ? 0.f : state[3 * i + 1],
           sd = first ? 0.f : state[3 * i + 2];
     float ca[kDC];
-    vsum_chunk(cax, am, x, y, X, (size_t)X * Y, min(dc, D - d0), ca);
+    vsum_chunk(hs, bs, am, x, y, X, ca);
 #pragma unroll
     for (int k = 0; k < kDC; ++k) {
-        if (k >= dc || d0 + k >= D) break;
+        if (d0 + k >= D) break;
         const float z = -(ca[k] * inv_n) * inv_tau;
         const float d = (float)(d0 + k);
         if (z > m) {
@@ -208,41 +278,42 @@ __global__ void diff_vagg_softmax_kernel(const float *__restrict__ cax, const ui
 
 // Backward 1: d dhat / d CA = p_d (d - dhat) (-1/tau) / n, times the
 // incoming gradient, for the chunk (the aggregated slab is recomputed).
-__global__ void diff_gca_kernel(const float *__restrict__ cax, const uint32_t *__restrict__ arm,
-                                const float *__restrict__ ns, int X, int Y, int D, int d0, int dc, float inv_tau,
-                                const float *__restrict__ dhat, const float *__restrict__ stats,
-                                const float *__restrict__ go, float *__restrict__ g0)
+__global__ void diff_gca_kernel(const float4 *__restrict__ hs, const float4 *__restrict__ bs,
+                                const uint32_t *__restrict__ arm, const float *__restrict__ ns, int X, int Y, int D,
+                                int d0, float inv_tau, const float *__restrict__ dhat, const float *__restrict__ stats,
+                                const float *__restrict__ go, float4 *__restrict__ g0)
 {
-    // 2-D tiles of kTileX x kTileY pixels: the warps of a block walk the
-    // same anchor rows, so their vertical windows meet in L1
+    pdl_trigger();
     const int x = blockIdx.x * kTileX + (int)(threadIdx.x % kTileX);
     const int y = blockIdx.y * kTileY + (int)(threadIdx.x / kTileX);
+    pdl_wait();
     if (x >= X || y >= Y) return;
     const int i = y * X + x;
     const size_t b = blockIdx.z, n = (size_t)X * Y;   // pair
-    cax += b * kDC * n;
+    hs += b * 2 * n;
+    bs += b * 2 * X * (size_t)((Y + 3) / 4);
     arm += b * n;
     ns += b * n;
     dhat += b * n;
     stats += b * 2 * n;
     go += b * n;
-    g0 += b * kDC * n;
+    g0 += b * 2 * n;
     const uint32_t am = arm[i];
     const float inv_n = 1.f / ns[i];
     const float m = stats[2 * i], s = stats[2 * i + 1], e = dhat[i], gi = go[i];
-    float ca[kDC];
-    vsum_chunk(cax, am, x, y, X, (size_t)X * Y, min(dc, D - d0), ca);
+    float ca[kDC], v[kDC];
+    vsum_chunk(hs, bs, am, x, y, X, ca);
 #pragma unroll
     for (int k = 0; k < kDC; ++k) {
-        if (k >= dc) break;
-        float v = 0.f;
+        v[k] = 0.f;
         if (d0 + k < D) {
             const float z = -(ca[k] * inv_n) * inv_tau;
             const float p = expf(z - m) / s;
-            v = gi * p * ((float)(d0 + k) - e) * (-inv_tau) * inv_n;
+            v[k] = gi * p * ((float)(d0 + k) - e) * (-inv_tau) * inv_n;
         }
-        g0[(size_t)k * X * Y + i] = v;
     }
+    g0[2 * (size_t)i] = make_float4(v[0], v[1], v[2], v[3]);
+    g0[2 * (size_t)i + 1] = make_float4(v[4], v[5], v[6], v[7]);
 }
 
 // Backward 2: adjoint of the vertical sum. G1(x, y') collects the anchors
@@ -257,25 +328,27 @@ constexpr int kVB = 32;
 static_assert(kDiffNT == 32 * kDC, "a block is 32 columns x the chunk's disparities");
 __global__ void __launch_bounds__(kDiffNT) diff_vT_kernel(const float *__restrict__ g0,
                                                           const uint32_t *__restrict__ arm, int X, int Y, int wy,
-                                                          int dc, float *__restrict__ g1)
+                                                          float *__restrict__ g1)
 {
     __shared__ float delta[kDiffNT][kVB + 1];     // odd pitch: the lanes of a warp hit distinct banks
-    const int xi = threadIdx.x % 32, k = threadIdx.x / 32;   // 32 columns x kDC disparities
+    pdl_trigger();
+    const int k = threadIdx.x % kDC, xi = threadIdx.x / kDC;   // 32 columns x kDC disparities
     const int x = blockIdx.x * 32 + xi, y0 = blockIdx.y * kVB;
-    if (x >= X || k >= dc) return;
+    pdl_wait();
+    if (x >= X) return;
     const size_t b = blockIdx.z, n = (size_t)X * Y;   // pair
-    arm += b * n;
-    const float *gp = g0 + b * kDC * n + (size_t)k * n + x;
-    float *out = g1 + b * kDC * n + (size_t)k * n + x;
+    arm += b * n + x;
+    const float *gp = g0 + (b * n + x) * kDC + k;
+    float *out = g1 + (b * n + x) * kDC + k;
     float *dl = delta[threadIdx.x];
     const int ye = min(y0 + kVB, Y);              // band rows [y0, ye)
 #pragma unroll
     for (int i = 0; i <= kVB; ++i) dl[i] = 0.f;
     const int ya = max(y0 - wy, 0), yb = min(ye - 1 + wy, Y - 1);
-#pragma unroll 4
+#pragma unroll 8
     for (int y = ya; y <= yb; ++y) {
-        const uint32_t am = arm[(size_t)y * X + x];
-        const float v = gp[(size_t)y * X];           // rows [ya, yb] are in the image: loaded ahead of the test
+        const uint32_t am = __ldg(arm + (size_t)y * X);
+        const float v = __ldg(gp + (size_t)y * X * kDC);   // rows [ya, yb] are in the image: loaded ahead of the test
         const int lo = y - (int)((am >> 16) & 0xFF), hi = y + (int)(am >> 24);
         if (hi >= y0 && lo < ye) {
             dl[max(lo, y0) - y0] += v;
@@ -285,167 +358,168 @@ __global__ void __launch_bounds__(kDiffNT) diff_vT_kernel(const float *__restric
     float s = 0.f;
     for (int i = 0; i < ye - y0; ++i) {
         s += dl[i];
-        out[(size_t)(y0 + i) * X] = s;
+        out[(size_t)(y0 + i) * X * kDC] = s;
     }
 }
 
-// Backward 3: adjoint of the horizontal sum. G2(x', y) collects the pixels
-// (x, y) whose own window [x - left, x + right] contains x'. A block takes one
-// row segment of up to kHSeg columns of one pair: it stages the chunk's
-// disparity planes and the arm words of the segment and its wx-column halo in
-// shared memory (coalesced loads), then, as in the vertical adjoint, a thread
-// owns one disparity and a band of 32 columns: each pixel whose window reaches
-// the band adds its value where the window enters and subtracts it one column
-// past where it ends (pixels in ascending x), and a running sum gives the
-// band. The staged rows skip a word every 32, so the 32 bands of a warp,
-// 32 columns apart, read distinct banks. The outputs go back through shared
-// memory and leave in coalesced rows.
-constexpr int kHSeg = 1024;                       // 32 bands of 32 columns
-__host__ __device__ __forceinline__ int hpad(int i) { return i + (i >> 5); }
+// Backward 3 and 4 in one: the adjoint of the horizontal sum, then through the
+// cost. A block takes one row segment of up to kHSeg - kDC + 1 columns of one
+// pair.
+//  * G2(x', y) collects the pixels (x, y) whose own window [x - left, x + right]
+//    contains x'. The chunk's G1 values and the arm words of the segment, its
+//    next kDC - 1 columns and a wx halo are staged in shared memory; a thread
+//    owns one disparity and a band of kHB columns: each pixel whose window
+//    reaches the band adds its value where the window enters and subtracts it
+//    one column past where it ends (pixels in ascending x), and a running sum
+//    gives the band. The staged columns skip one every 16, so that the bands of
+//    a warp read distinct banks.
+//  * A cell (x, y, d) passes v = G2 dC/dgL to its left pixel and -v to the right
+//    pixel x - d: v goes through shared memory, and the block takes the right
+//    pixels whose cells of this chunk all lie in its columns. The four
+//    parameters get one partial per block, summed later in a fixed order.
+constexpr int kHSeg = 512, kHB = 16;
+static_assert(kHSeg / kHB * kDC == kDiffNT, "one (band, disparity) per thread");
+__host__ __device__ __forceinline__ int hpad(int i) { return i + (i >> 4); }
+__host__ __device__ __forceinline__ int hgrad_segments(int X) { return (X + kHSeg - kDC) / (kHSeg - kDC + 1); }
 
-size_t diff_hT_smem(int X, int wx)
+size_t diff_hgrad_smem(int wx)
 {
-    const int seg = min(X, kHSeg), span = seg + 2 * wx;
-    return (size_t)(kDC + 1) * hpad(span + 31) * 4 + (size_t)kDiffNT * 33 * 4;
+    const int span = hpad(kHSeg + 2 * wx) + 1;
+    return (size_t)span * kDC * 4 + (size_t)span * 4 + (size_t)kDiffNT * (kHB + 1) * 4;
 }
+static_assert(kDiffNT * (kHB + 1) >= kDC * kHSeg, "the difference arrays' space takes the cells' values");
 
-__global__ void __launch_bounds__(kDiffNT) diff_hT_kernel(const float *__restrict__ g1,
-                                                          const uint32_t *__restrict__ arm, int X, int Y, int wx,
-                                                          int dc, float *__restrict__ g2)
+__global__ void __launch_bounds__(kDiffNT) diff_hgrad_kernel(
+    const float *__restrict__ g1, const uint32_t *__restrict__ arm, const float *__restrict__ gL,
+    const float *__restrict__ gR, const uint32_t *__restrict__ pixL, const uint32_t *__restrict__ pixR,
+    const float *__restrict__ theta, int X, int Y, int D, int d0, int wx, int rows, int first,
+    float *__restrict__ acc_l, float *__restrict__ acc_r, float *__restrict__ part, size_t part_pair)
 {
-    extern __shared__ float hsm[];
-    const int seg = min(X, kHSeg), span = seg + 2 * wx, pitch = hpad(span + 31);
-    float *gs = hsm;                                          // [kDC][pitch] staged planes, then outputs
-    uint32_t *as = reinterpret_cast<uint32_t *>(hsm + kDC * pitch);   // [pitch] arm words
-    float *delta = hsm + (kDC + 1) * pitch;                   // [kDiffNT][33]
-    const int y = blockIdx.y, x0 = blockIdx.x * kHSeg;
-    const int xs = x0 - wx;                                   // column of staged index 0
-    const int x1 = min(x0 + kHSeg, X);                        // segment columns [x0, x1)
+    extern __shared__ __align__(16) float hsm[];
+    __shared__ float eh_t[8];
+    __shared__ float sh[4][kDiffNT / 32];
+    pdl_trigger();
+    const int span = hpad(kHSeg + 2 * wx) + 1;
+    float *gs = hsm;                                          // [span][kDC] staged G1, then G2
+    uint32_t *as = reinterpret_cast<uint32_t *>(hsm + span * kDC);   // [span] arm words
+    float *delta = hsm + span * (kDC + 1);                    // [kDiffNT][kHB + 1], then v [kDC][kHSeg]
+    const int nseg = hgrad_segments(X), seg = (X + nseg - 1) / nseg;
+    const int s0 = blockIdx.x * seg, s1 = min(s0 + seg, X);   // the segment's left pixels
+    const int s2 = min(s1 + kDC - 1, X);                      // the columns whose cells it needs
+    const int xs = s0 - wx;                                   // column of staged index 0
     const size_t b = blockIdx.z, n = (size_t)X * Y;           // pair
-    const size_t r = (size_t)y * X;
+    pdl_wait();
     g1 += b * kDC * n;
-    g2 += b * kDC * n;
     arm += b * n;
-    // stage the planes and arms of columns [max(xs, 0), min(x1 + wx, X))
-    const int sa = max(xs, 0), sb = min(x1 + wx, X);
-    for (int x = sa + (int)threadIdx.x; x < sb; x += kDiffNT) {
-        as[hpad(x - xs)] = arm[r + x];
-        for (int k = 0; k < dc; ++k) gs[k * pitch + hpad(x - xs)] = g1[(size_t)k * n + r + x];
-    }
-    __syncthreads();
-    const int k = threadIdx.x / 32, band = threadIdx.x % 32;
-    const int bx0 = x0 + 32 * band;                           // band columns [bx0, be)
-    const int be = min(bx0 + 32, x1);
-    float *dl = delta + threadIdx.x * 33;
-    float acc[32];
-    const bool work = k < dc && bx0 < be;
-    if (work) {
-#pragma unroll
-        for (int i = 0; i <= 32; ++i) dl[i] = 0.f;
-        const float *gk = gs + k * pitch;
-        const int xa = max(bx0 - wx, 0), xb = min(be - 1 + wx, X - 1);
-        for (int x = xa; x <= xb; ++x) {
-            const uint32_t am = as[hpad(x - xs)];
-            const int lo = x - (int)(am & 0xFF), hi = x + (int)((am >> 8) & 0xFF);
-            if (hi < bx0 || lo >= be) continue;
-            const float v = gk[hpad(x - xs)];
-            dl[max(lo, bx0) - bx0] += v;
-            if (hi + 1 < be) dl[hi + 1 - bx0] -= v;
-        }
-        float sacc = 0.f;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            sacc += dl[i];
-            acc[i] = sacc;
-        }
-    }
-    __syncthreads();                              // every thread is done with the staged planes
-    if (work)
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (bx0 + i < be) gs[k * pitch + hpad(bx0 + i - xs)] = acc[i];
-    __syncthreads();
-    for (int x = x0 + (int)threadIdx.x; x < x1; x += kDiffNT)
-        for (int kk = 0; kk < dc; ++kk) g2[(size_t)kk * n + r + x] = gs[kk * pitch + hpad(x - xs)];
-}
-
-// Backward 4: through the cost. Per pixel: its own gradient as the left pixel
-// of every cell (x, y, d), as the right pixel x' of the cells (x' + d, y, d),
-// and its cells' contributions to the four parameters (one partial per block,
-// summed later in a fixed order).
-__global__ void diff_costgrad_kernel(const float *__restrict__ gL, const float *__restrict__ gR,
-                                     const uint32_t *__restrict__ pixL, const uint32_t *__restrict__ pixR,
-                                     const float *__restrict__ theta, int X, int Y, int D, int d0, int dc,
-                                     const float *__restrict__ g2, float *__restrict__ acc_l,
-                                     float *__restrict__ acc_r, float *__restrict__ part, size_t part_pair)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t b = blockIdx.y, n = (size_t)X * Y;   // pair
     gL += b * n;
     gR += b * n;
     pixL += b * n;
     pixR += b * n;
-    g2 += b * kDC * n;
     acc_l += b * n;
     acc_r += b * n;
-    part += b * part_pair;
     const Theta th = load_theta(theta);
     const float inv_lad = 1.f / th.lad, inv_lmc = 1.f / th.lmc;
     const float kad = th.wad * inv_lad;                 // w_AD / l_AD
     const float dad = th.wad * inv_lad * inv_lad;       // w_AD / l_AD^2
     const float dmc = th.wmc * inv_lmc * inv_lmc;       // w_MC / l_MC^2
     // exp(-h / l_MC) for the seven Hamming distances
-    __shared__ float eh_t[8];
     if (threadIdx.x < 7) eh_t[threadIdx.x] = expf(-(float)threadIdx.x * inv_lmc);
-    __syncthreads();
+    const float ea1 = expf(-inv_lad);
+    const int kn = min(kDC, D - d0);
     float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f;
-    if (i < X * Y) {
-        const int y = i / X, x = i - y * X;
+    for (int y = blockIdx.y * rows; y < min(((int)blockIdx.y + 1) * rows, Y); ++y) {
         const size_t r = (size_t)y * X;
-        const int kn = min(dc, D - d0);
-        const float gl = gL[i], gr = gR[i];
-        const uint32_t pl = pixL[i];
-        const float ea1 = expf(-inv_lad), eh6 = eh_t[6];   // the terms of P (|a| = 1, h = 6)
-        float al = 0.f, ar = 0.f;
-        // the chunk's disparities unrolled, so their loads and exps overlap
+        __syncthreads();                                      // the previous row is done with shared memory
+        const int sa = max(xs, 0), sb = min(s2 + wx, X);
+        for (int i = threadIdx.x; i < (sb - sa) * 2; i += kDiffNT) {
+            const int x = sa + (i >> 1);
+            reinterpret_cast<float4 *>(gs)[hpad(x - xs) * 2 + (i & 1)] =
+                __ldg(reinterpret_cast<const float4 *>(g1) + (r + x) * 2 + (i & 1));
+        }
+        for (int x = sa + (int)threadIdx.x; x < sb; x += kDiffNT) as[hpad(x - xs)] = __ldg(arm + r + x);
+        __syncthreads();
+        {
+            const int k = threadIdx.x % kDC, bx0 = s0 + kHB * (int)(threadIdx.x / kDC);
+            const int be = min(bx0 + kHB, s2);                // band columns [bx0, be)
+            float *dl = delta + threadIdx.x * (kHB + 1);
+            float acc[kHB];
+            const bool work = bx0 < be;
+            if (work) {
 #pragma unroll
-        for (int k = 0; k < kDC; ++k) {
-            if (k < kn) {
-                const int d = d0 + k;
-                const float *plane = g2 + (size_t)k * X * Y;
-                const float g = plane[i];
-                if (x < d) {
-                    t0 += g * (1.f - ea1);
-                    t1 += g * (1.f - eh6);
-                    t2 += g * (-ea1 * dad);
-                    t3 += g * (-eh6 * 6.f * dmc);
-                } else {
-                    const float diff = gl - gR[i - d], a = fabsf(diff);
-                    const int hi = __popc((pl ^ pixR[i - d]) & 0x3F00u);
-                    const float h = (float)hi;
-                    const float ea = expf(-a * inv_lad), eh = eh_t[hi];
-                    t0 += g * (1.f - ea);
-                    t1 += g * (1.f - eh);
-                    t2 += g * (-ea * a * dad);
-                    t3 += g * (-eh * h * dmc);
-                    const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
-                    al += g * kad * ea * sgn;
+                for (int i = 0; i <= kHB; ++i) dl[i] = 0.f;
+                const int xa = max(bx0 - wx, 0), xb = min(be - 1 + wx, X - 1);
+#pragma unroll 4
+                for (int x = xa; x <= xb; ++x) {
+                    const uint32_t am = as[hpad(x - xs)];
+                    const float v = gs[hpad(x - xs) * kDC + k];
+                    const int lo = x - (int)(am & 0xFF), hi = x + (int)((am >> 8) & 0xFF);
+                    if (hi >= bx0 && lo < be) {
+                        dl[max(lo, bx0) - bx0] += v;
+                        if (hi + 1 < be) dl[hi + 1 - bx0] -= v;
+                    }
                 }
-                // this pixel as the match of the left pixel x + d
-                if (x + d < X) {
-                    const float gg = plane[r + x + d];
-                    const float diff = gL[r + x + d] - gr, a = fabsf(diff);
-                    const float ea = expf(-a * inv_lad);
-                    const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
-                    ar -= gg * kad * ea * sgn;
+                float s = 0.f;
+#pragma unroll
+                for (int i = 0; i < kHB; ++i) {
+                    s += dl[i];
+                    acc[i] = s;
                 }
             }
+            __syncthreads();                                  // every thread is done with the staged values
+            if (work)
+#pragma unroll
+                for (int i = 0; i < kHB; ++i)
+                    if (bx0 + i < be) gs[hpad(bx0 + i - xs) * kDC + k] = acc[i];
         }
-        acc_l[i] += al;
-        acc_r[i] += ar;
+        __syncthreads();
+        for (int x = s0 + (int)threadIdx.x; x < s2; x += kDiffNT) {
+            const float gl = gL[r + x];
+            const uint32_t pl = pixL[r + x];
+            const float4 ga = *reinterpret_cast<const float4 *>(gs + hpad(x - xs) * kDC);
+            const float4 gb = *reinterpret_cast<const float4 *>(gs + hpad(x - xs) * kDC + 4);
+            const float g[kDC] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+            const bool own = x < s1;
+            float al = 0.f;
+            // the chunk's disparities unrolled, so their loads and exps overlap
+#pragma unroll
+            for (int k = 0; k < kDC; ++k) {
+                const int d = d0 + k;
+                float v = 0.f;
+                if (k < kn) {
+                    float ea = ea1, a = 1.f;                  // the terms of P (|a| = 1, h = 6)
+                    int h = 6;
+                    if (x >= d) {
+                        const float diff = gl - gR[r + x - d];
+                        a = fabsf(diff);
+                        h = __popc((pl ^ pixR[r + x - d]) & 0x3F00u);
+                        ea = expf(-a * inv_lad);
+                        const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
+                        v = g[k] * kad * ea * sgn;
+                    }
+                    if (own) {
+                        const float eh = eh_t[h];
+                        t0 += g[k] * (1.f - ea);
+                        t1 += g[k] * (1.f - eh);
+                        t2 += g[k] * (-ea * a * dad);
+                        t3 += g[k] * (-eh * (float)h * dmc);
+                        al += v;
+                    }
+                }
+                delta[k * kHSeg + x - s0] = v;
+            }
+            if (own) acc_l[r + x] = first ? al : acc_l[r + x] + al;
+        }
+        __syncthreads();
+        // right pixel x is the match of the left pixels x + d0 .. x + d0 + kn - 1
+        for (int x = max(s0 - d0, 0) + (int)threadIdx.x; x < s1 - d0; x += kDiffNT) {
+            float ar = 0.f;
+#pragma unroll
+            for (int k = 0; k < kDC; ++k)
+                if (x + d0 + k < s2) ar -= delta[k * kHSeg + x + d0 + k - s0];
+            acc_r[r + x] = first ? ar : acc_r[r + x] + ar;
+        }
     }
     // block partials of the parameter gradients
-    __shared__ float sh[4][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -463,8 +537,8 @@ __global__ void diff_costgrad_kernel(const float *__restrict__ gL, const float *
     __syncthreads();
     if (threadIdx.x < 4) {
         float s = 0.f;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += sh[threadIdx.x][k];
-        part[(size_t)blockIdx.x * 4 + threadIdx.x] = s;
+        for (int k = 0; k < kDiffNT / 32; ++k) s += sh[threadIdx.x][k];
+        part[b * part_pair + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + threadIdx.x] = s;
     }
 }
 
@@ -597,14 +671,11 @@ size_t diff_workspace_bytes(int X, int Y, int wy, int B, int D)
 
 cudaError_t diff_setup()
 {
-    // the cost rows of a chunk take up to kDC * 4096 floats of shared memory;
-    // the horizontal adjoint stages a 1024-column segment with a halo of up to
-    // 141 columns each side
     cudaError_t e = cudaFuncSetAttribute(diff_costx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kDC * 4096 * (int)sizeof(float));
+                                         (int)diff_costx_smem(4096, kMaxWx));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(diff_hT_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)diff_hT_smem(kHSeg, kMaxWx));
+    return cudaFuncSetAttribute(diff_hgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)diff_hgrad_smem(kMaxWx));
 }
 
 cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
@@ -614,7 +685,16 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
     diff_layout((char *)a.ws, X, Y, a.wy, B, a.D, &w);
     const int nblk = (n + kDiffNT - 1) / kDiffNT;
     const int nchunks = (a.D + kDC - 1) / kDC;
-    const size_t part_pair = (size_t)nchunks * nblk * 4;
+    // parameter-gradient partials, one per block of the cost gradient: they
+    // take the planes [armr, ns) that this form leaves unused, with more rows
+    // to a block where a narrow image's would not hold them
+    const size_t room = (size_t)((char *)w.ns - (char *)w.armr);
+    const int nseg = hgrad_segments(X);
+    int rows = 1;
+    while ((size_t)B * nchunks * nseg * ((Y + rows - 1) / rows) * 16 > room) ++rows;
+    const int yblocks = (Y + rows - 1) / rows;
+    float *part = (float *)w.armr;
+    const size_t part_chunk = (size_t)nseg * yblocks * 4, part_pair = part_chunk * nchunks;
     const float inv_tau = 1.f / a.tau;
     const dim3 tiles((X + kTileX - 1) / kTileX, (Y + kTileY - 1) / kTileY, B);
     static_assert(kTileX * kTileY == kDiffNT, "one thread per pixel of a tile");
@@ -622,11 +702,7 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
     // frozen supports of every pair (integer path), support sizes, float grey
     diff_grey_kernel<<<dim3(nblk, 2, B), kDiffNT, 0, s>>>(a.left, a.right, w.gl, w.gr, n);
     // (the arms of the left images only: nothing here uses the right base)
-    for (int b = 0; b < B; ++b) {
-        const size_t o = (size_t)b * n;
-        if ((e = launch_grey(a.left_u8 + o * 3, a.right_u8 + o * 3, w.ql + o, w.qr + o, X, Y, s)) != cudaSuccess)
-            return e;
-    }
+    if ((e = launch_grey(a.left_u8, a.right_u8, w.ql, w.qr, X, Y * B, s)) != cudaSuccess) return e;
     for (int b0 = 0; b0 < B; b0 += kMaxSupImages / 2) {
         SupImage im[kMaxSupImages];
         const int nb = min(B - b0, kMaxSupImages / 2);
@@ -638,35 +714,31 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
         if ((e = launch_support(im, 2 * nb, a.wx, a.wy, a.tc, a.err, s)) != cudaSuccess) return e;
     }
     diff_nsupport_kernel<<<dim3(nblk, B), kDiffNT, 0, s>>>(w.arml, X, Y, w.ns);
-    if (a.backward) {
-        if ((e = cudaMemsetAsync(w.accl, 0, (size_t)B * n * 4, s)) != cudaSuccess ||
-            (e = cudaMemsetAsync(w.accr, 0, (size_t)B * n * 4, s)) != cudaSuccess)
-            return e;
-    }
-    for (int c = 0; c < nchunks; ++c) {
-        const int d0 = c * kDC, dc = min(kDC, a.D - d0);
-        diff_costx_kernel<<<dim3(Y, B), kDiffNT, (size_t)dc * X * 4, s>>>(w.gl, w.gr, w.pixl, w.pixr, w.arml,
-                                                                          a.theta, X, Y, a.D, d0, dc, w.s0);
+    float4 *hs = (float4 *)w.s0, *bs = (float4 *)w.s3;   // x sums, their row-quad sums
+    const dim3 cgrid((X + kCXSeg - 1) / kCXSeg, (Y + 3) / 4, B);
+    for (int c = 0; c < nchunks && e == cudaSuccess; ++c) {
+        const int d0 = c * kDC;
+        e = launch_dependent(diff_costx_kernel, cgrid, dim3(kDiffNT), diff_costx_smem(X, a.wx), s, w.gl, w.gr, w.pixl,
+                             w.pixr, w.arml, a.theta, X, Y, a.D, d0, a.wx, hs, bs);
+        if (e != cudaSuccess) break;
         if (!a.backward) {
-            diff_vagg_softmax_kernel<<<tiles, kDiffNT, 0, s>>>(w.s0, w.arml, w.ns, X, Y, a.D, d0, dc,
-                                                                       inv_tau, w.state, c == 0, c == nchunks - 1,
-                                                                       a.dhat, a.stats);
-        } else {
-            diff_gca_kernel<<<tiles, kDiffNT, 0, s>>>(w.s0, w.arml, w.ns, X, Y, a.D, d0, dc, inv_tau,
-                                                              a.dhat, a.stats, a.grad_dhat, w.s1);
-            diff_vT_kernel<<<dim3((X + 31) / 32, (Y + kVB - 1) / kVB, B), kDiffNT, 0, s>>>(w.s1, w.arml, X, Y,
-                                                                                      a.wy, dc, w.s2);
-            diff_hT_kernel<<<dim3((X + kHSeg - 1) / kHSeg, Y, B), kDiffNT, diff_hT_smem(X, a.wx), s>>>(
-                w.s2, w.arml, X, Y, a.wx, dc, w.s3);
-            diff_costgrad_kernel<<<dim3(nblk, B), kDiffNT, 0, s>>>(w.gl, w.gr, w.pixl, w.pixr, a.theta, X, Y, a.D,
-                                                                   d0, dc, w.s3, w.accl, w.accr,
-                                                                   w.part + (size_t)c * nblk * 4, part_pair);
+            e = launch_dependent(diff_vagg_softmax_kernel, tiles, dim3(kDiffNT), 0, s, hs, bs, w.arml, w.ns, X, Y, a.D,
+                                 d0, inv_tau, w.state, c == 0, c == nchunks - 1, a.dhat, a.stats);
+            continue;
         }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_dependent(diff_gca_kernel, tiles, dim3(kDiffNT), 0, s, hs, bs, w.arml, w.ns, X, Y, a.D, d0,
+                                  inv_tau, a.dhat, a.stats, a.grad_dhat, (float4 *)w.s1)) != cudaSuccess ||
+            (e = launch_dependent(diff_vT_kernel, dim3((X + 31) / 32, (Y + kVB - 1) / kVB, B), dim3(kDiffNT), 0, s,
+                                  w.s1, w.arml, X, Y, a.wy, w.s2)) != cudaSuccess)
+            break;
+        e = launch_dependent(diff_hgrad_kernel, dim3(nseg, yblocks, B), dim3(kDiffNT), diff_hgrad_smem(a.wx), s, w.s2,
+                             w.arml, w.gl, w.gr, w.pixl, w.pixr, a.theta, X, Y, a.D, d0, a.wx, rows, c == 0, w.accl,
+                             w.accr, part + c * part_chunk, part_pair);
     }
+    if (e != cudaSuccess) return e;
     if (a.backward) {
         diff_finish_kernel<<<dim3(nblk, B), kDiffNT, 0, s>>>(w.accl, w.accr, n, a.grad_left, a.grad_right);
-        diff_theta_segments_kernel<<<kRedBlocks, kRedNT, 0, s>>>(w.part, B * nchunks * nblk, w.seg);
+        diff_theta_segments_kernel<<<kRedBlocks, kRedNT, 0, s>>>(part, (int)(part_pair / 4 * B), w.seg);
         diff_theta_reduce_kernel<<<1, kRedNT, 0, s>>>(w.seg, a.grad_theta);
     }
     return cudaGetLastError();
