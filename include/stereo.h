@@ -229,7 +229,7 @@ typedef struct {
  * frame, the fused cost + aggregation + WTA of all frames runs as one
  * persistent kernel taking (frame, strip, slab) tiles largest frame first;
  * the whole batch is one CUDA graph, re-captured and updated in place on each
- * call. Each frame's maps equal stereo_compute's for that frame exactly.
+ * call (batches of up to four frames are launched directly). Each frame's maps equal stereo_compute's for that frame exactly.
  * With the automatic tile (stereo_set_tile(-1)) the first batch of a given
  * signature (frame shapes, parameters, GPU) times every tile shape that fits
  * and remembers the fastest; stereo_tune_save / stereo_tune_load keep those

@@ -744,19 +744,23 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
 {
     for (int j = 0; j < b.njobs; ++j)
         if (!fits<T>(b.job[j])) return cudaErrorInvalidValue;
-    // bands only where the frames' tiles leave SMs idle: the sum of all row
-    // steps over the SMs, and the longest tile at the end
+    // bands where the frames' tiles leave SMs idle: few tiles go in rounds over
+    // the SMs, many even out and leave about half a long tile at the end
     double best = 0;
     int nb = 1;
     for (int n = 1; n <= kMaxBands; ++n) {
         double sum = 0, last = 0;
+        long tiles = 0;
         for (int j = 0; j < b.njobs; ++j) {
             const CostAggArgs &a = b.job[j];
             const int rows = band_rows(a, n), steps = band_steps(a, rows);
-            sum += (double)tiles_of<T>(a) * ((a.Y + rows - 1) / rows) * steps;
+            const long nt = (long)tiles_of<T>(a) * ((a.Y + rows - 1) / rows);
+            tiles += nt;
+            sum += (double)nt * steps;
             last = std::max(last, (double)steps);
         }
-        const double t = std::max(sum / nsm, last) + 0.5 * last;
+        const double rounds = (double)((tiles + nsm - 1) / nsm);
+        const double t = std::max(last, rounds < 4 ? rounds * sum / tiles : sum / nsm + 0.5 * last);
         if (n == 1 || t < best) {
             best = t;
             nb = n;

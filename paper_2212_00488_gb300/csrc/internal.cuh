@@ -127,15 +127,17 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s);
 // Launchers (each returns the launch error, cudaSuccess on success).
 cudaError_t launch_grey(const uint8_t *rgb_l, const uint8_t *rgb_r, uint8_t *g_l, uint8_t *g_r,
                         int W, int H, cudaStream_t s);
-// Grey of both images and its Eq. 2 downscale, with the full-resolution grey
-// of the left image (what the scale-up reads): one launch when W is a
-// multiple of 4 and the RGB rows are word-aligned (gf_r is then not written),
-// else grey_kernel and downscale_kernel. Adds the kernels launched to
-// *launches.
-cudaError_t launch_grey_down(const uint8_t *rgb_l, const uint8_t *rgb_r, uint8_t *gf_l, uint8_t *gf_r,
-                            uint8_t *s_l, uint8_t *s_r, int W, int H, cudaStream_t s, int *launches);
-cudaError_t launch_downscale(const uint8_t *g_l, const uint8_t *g_r, uint8_t *s_l, uint8_t *s_r,
-                             int W, int H, cudaStream_t s);
+// Grey of both images of up to kMaxBatch frames and its Eq. 2 downscale, with
+// the full-resolution grey of the left image (what the scale-up reads): one launch
+// for the frames whose rows are word-aligned, one for the others. Adds the
+// kernels launched to *launches.
+struct GreyJob {
+    const uint8_t *rgb_l, *rgb_r;      // [H][W][3]
+    uint8_t *gf_l;                     // [H][W]
+    uint8_t *s_l, *s_r;                // [H / 2][W / 2]
+    int W, H;
+};
+cudaError_t launch_grey_down(const GreyJob *jobs, int n, cudaStream_t s, int *launches);
 // Mini-census codes and cross arms of up to kMaxSupImages images in one launch
 // (nx is filled by the launcher). Also presets the WTA keys to ~0 where key is
 // given, and clears the fused kernel's error word.
@@ -148,14 +150,19 @@ struct SupImage {
 };
 cudaError_t launch_support(const SupImage *im, int n, int wx, int wy, int tc, uint32_t *err, cudaStream_t s);
 cudaError_t launch_costagg(const CostAggArgs &a, cudaStream_t s);
-cudaError_t launch_refine(const uint32_t *key_l, const uint32_t *key_r, const uint8_t *grey_l,
-                          int X, int Y, int T, int fill_mode, uint8_t *dl, uint8_t *dr, uint8_t *gcp,
-                          uint8_t *dm, float *dplus, cudaStream_t s);
-// The downscaling path's Steps 6-8 in one kernel: the maps and dplus of
-// launch_refine, and the full-resolution disparity in out.
-cudaError_t launch_refine_up(const uint32_t *key_l, const uint32_t *key_r, const uint8_t *grey_low,
-                             const uint8_t *grey_full, int X, int Y, int W, int H, int T, int fill_mode, uint8_t *dl,
-                             uint8_t *dr, uint8_t *gcp, uint8_t *dm, float *dplus, float *out, cudaStream_t s);
+// Cross-check, median and fill (Steps 6-7) of up to kMaxBatch frames in one
+// launch, with up the scale-up (Step 8) in the same kernel. dl, dr, gcp, dm, dplus
+// may be null; without up, W, H, gf and out are not used.
+struct RefineJob {
+    const uint32_t *key_l, *key_r;     // [Y][X]
+    const uint8_t *gs, *gf;            // processed and full-resolution grey of the left image
+    int X, Y, W, H;
+    uint8_t *dl, *dr, *gcp, *dm;       // [Y][X]
+    float *dplus;                      // [Y][X]
+    float *out;                        // [H][W]
+    int pairs;                         // filled by the launcher
+};
+cudaError_t launch_refine(const RefineJob *jobs, int n, bool up, int T, int fill_mode, cudaStream_t s);
 cudaError_t launch_unpack_planes(const uint32_t *pix, const uint32_t *arm, uint8_t *grey,
                                  uint8_t *census, uint32_t *arms, int X, int Y, cudaStream_t s);
 

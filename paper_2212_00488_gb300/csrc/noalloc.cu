@@ -121,8 +121,8 @@ extern "C" int stereo_compute_noalloc(const stereo_params *params, const uint8_t
     float *dplus = ds ? reinterpret_cast<float *>(base + o_dplus) : disp_out;
 
     int launches = 0;
-    if ((e = ds ? launch_grey_down(left_rgb, right_rgb, u8(o_gf[0]), u8(o_gf[1]), u8(o_gs[0]), u8(o_gs[1]), W, H,
-                                   s, &launches)
+    const GreyJob grey{left_rgb, right_rgb, u8(o_gf[0]), u8(o_gs[0]), u8(o_gs[1]), W, H};
+    if ((e = ds ? launch_grey_down(&grey, 1, s, &launches)
                 : launch_grey(left_rgb, right_rgb, u8(o_gf[0]), u8(o_gf[1]), W, H, s)) == cudaSuccess &&
         (e = [&] {
             SupImage im[2];
@@ -154,10 +154,11 @@ extern "C" int stereo_compute_noalloc(const stereo_params *params, const uint8_t
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         a.num_sms = nsm;
         if ((e = launch_costagg(a, s)) == cudaSuccess)
-            e = ds ? launch_refine_up(u32(o_key[0]), u32(o_key[1]), u8(o_gs[0]), u8(o_gf[0]), X, Y, W, H, p.t_fill,
-                                      p.fill_mode, dl_out, dr_out, gcp_out, u8(o_dm), dplus, disp_out, s)
-                   : launch_refine(u32(o_key[0]), u32(o_key[1]), u8(o_gs[0]), X, Y, p.t_fill, p.fill_mode, dl_out, dr_out,
-                                   gcp_out, u8(o_dm), dplus, s);
+        {
+            const RefineJob j{u32(o_key[0]), u32(o_key[1]), u8(o_gs[0]), u8(o_gf[0]), X, Y, W, H, dl_out, dr_out,
+                              gcp_out, u8(o_dm), dplus, disp_out, 0};
+            e = launch_refine(&j, 1, ds, p.t_fill, p.fill_mode, s);
+        }
     }
     if (e != cudaSuccess) return say(err, err_len, STEREO_ECUDA, "kernel launch: %s", cudaGetErrorString(e));
     return STEREO_OK;

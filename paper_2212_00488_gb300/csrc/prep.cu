@@ -51,70 +51,86 @@ __global__ void grey_kernel(const uint8_t *__restrict__ rgb_l, const uint8_t *__
     }
 }
 
-// Eq. 2 with K = 2, m = 1: mean of the 3x3 window centred on (2x, 2y),
-// coordinates clamped to the image, rounded half up: (sum + 4) / 9.
-__global__ void downscale_kernel(const uint8_t *__restrict__ g_l, const uint8_t *__restrict__ g_r,
-                                 uint8_t *__restrict__ s_l, uint8_t *__restrict__ s_r, int W, int H)
-{
-    const uint8_t *g = blockIdx.z ? g_r : g_l;
-    uint8_t *s = blockIdx.z ? s_r : s_l;
-    int X = W / 2, Y = H / 2;
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y;
-    if (x >= X || y >= Y) return;
-    int sum = 0;
-#pragma unroll
-    for (int j = -1; j <= 1; ++j) {
-        int yy = min(max(2 * y + j, 0), H - 1);
-        const uint8_t *row = g + (size_t)yy * W;
-#pragma unroll
-        for (int i = -1; i <= 1; ++i) sum += __ldg(row + min(max(2 * x + i, 0), W - 1));
-    }
-    s[(size_t)y * X + x] = (uint8_t)((sum + 4) / 9);
-}
-
-// Grey conversion and Eq. 2 downscale in one pass (the downscaling path, for
-// W a multiple of 4 and 4-byte aligned RGB rows). Thread (band, c) of one
-// image owns full-res columns 4c .. 4c + 3 and makes the 3x3 means of output
-// columns 2c, 2c + 1, rows 4 band .. 4 band + 3. It converts rows
-// 8 band - 1 .. 8 band + 7 of its columns (row coordinates clamped, as in
-// downscale_kernel), each from three aligned words, all requested before the
-// first is used; the grey of pixel 4c - 1 comes from the word its left
-// neighbour loaded (a shuffle; lane 0 loads it itself). Grey values stay in
-// registers; the left image's full-res grey of rows 8 band .. 8 band + 7 is
-// written for the scale-up. Bands cover ceil(H / 2) rows so that the last row
-// of an odd H gets its grey. Same arithmetic as grey_kernel followed by
-// downscale_kernel.
+// Grey conversion and Eq. 2 downscale in one pass (the downscaling path): with K =
+// 2, m = 1 the mean of the 3x3 window centred on (2x, 2y), coordinates clamped to
+// the image, rounded half up: (sum + 4) / 9. Thread (band, c) of one image owns
+// full-res columns 4c .. 4c + 3 and makes the means of output columns 2c, 2c + 1, rows
+// 4 band .. 4 band + 3. It converts rows 8 band - 1 .. 8 band + 7 of its columns (row
+// coordinates clamped), each from three words, all requested before the first is
+// used; the grey of pixel 4c - 1 comes from its left neighbour (a shuffle; lane 0
+// loads it itself). A window's last column 2x + 1 always lies in the image. Grey
+// values stay in registers; the left image's full-res grey of rows 8 band .. 8
+// band + 7 is written for the scale-up. Bands cover ceil(H / 2) rows so that the
+// last row of an odd H gets its grey.
+//
+// kAligned: W a multiple of 4 and word-aligned rows. Else a row's words are funnel
+// shifts of the aligned words that hold its pixels, the last group of a row may
+// be partial, and stores go by halfwords or bytes (1482 x 994: 10.3 us as two
+// kernels, 8.8 now). The frames of a batch share a launch of each kind.
 constexpr int kGDT = 128;                  // threads per CTA
 constexpr int kGDB = 4;                    // output rows per thread
 constexpr int kGDR = 2 * kGDB + 1;         // full-res rows per thread
 
-__global__ void __launch_bounds__(kGDT) grey_down_kernel(
-    const uint8_t *__restrict__ rgb_l, const uint8_t *__restrict__ rgb_r, uint8_t *__restrict__ gf_l,
-    uint8_t *__restrict__ s_l, uint8_t *__restrict__ s_r, int W, int H, int ncol, int nband)
+template <int N>
+struct GreyArgs {
+    int n;
+    int start[N + 1];                      // first CTA of each image (two per frame)
+    GreyJob job[N / 2];
+};
+
+template <bool kAligned, int N>
+__global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__ GreyArgs<N> A)
 {
     pdl_trigger();
-    pdl_wait();   // launched early behind the previous frame's last kernel, which still reads gf and s
-    const bool right = blockIdx.y != 0;
-    const int t0 = blockIdx.x * kGDT + threadIdx.x;
-    const int nthr = ncol * nband;
+    int im = 0;
+    while (im + 1 < A.n && (int)blockIdx.x >= A.start[im + 1]) ++im;
+    const GreyJob &J = A.job[im >> 1];
+    const bool right = im & 1;
+    const int W = J.W, H = J.H, X = W / 2, Y = H / 2;
+    const int ncol = (W + 3) / 4, nthr = ncol * (((H + 1) / 2 + kGDB - 1) / kGDB);
+    const int t0 = ((int)blockIdx.x - A.start[im]) * kGDT + threadIdx.x;
     // threads past the end take the last thread's pixels for the shuffles
     // and store nothing
     const bool live = t0 < nthr;
     const int t = live ? t0 : nthr - 1;
     const int band = t / ncol, c = t - band * ncol;   // left neighbour (band, c - 1) is thread t - 1
     const int lane = threadIdx.x & 31;
-    const uint8_t *rgb = right ? rgb_r : rgb_l;
-    uint8_t *s = right ? s_r : s_l;
-    const int X = W / 2, Y = H / 2;
+    const uint8_t *rgb = right ? J.rgb_r : J.rgb_l;
+    uint8_t *s = right ? J.s_r : J.s_l, *gf = J.gf_l;
+    const int nc = min(4, W - 4 * c);                 // columns of the group
+    pdl_wait();   // launched early behind the previous frame's last kernel, which still reads gf and s
     uint32_t w[kGDR][3], wh[kGDR];
 #pragma unroll
     for (int r = 0; r < kGDR; ++r) {
         const int fy = min(max(8 * band - 1 + r, 0), H - 1);
-        const uint32_t *p = reinterpret_cast<const uint32_t *>(rgb + ((size_t)fy * W + 4 * c) * 3);
+        const uint8_t *p = rgb + ((size_t)fy * W + 4 * c) * 3;
+        if (kAligned) {
+            const uint32_t *q = reinterpret_cast<const uint32_t *>(p);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) w[r][i] = __ldg(p + i);
-        wh[r] = lane == 0 && c > 0 ? __ldg(p - 1) : 0u;
+            for (int i = 0; i < 3; ++i) w[r][i] = __ldg(q + i);
+            wh[r] = lane == 0 && c > 0 ? __ldg(q - 1) : 0u;
+        } else {
+            // whole groups whose last word ends inside the image's bytes
+            const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3) * 8;
+            if (nc == 4 && (fy + 1 < H || 4 * c + 8 <= W)) {
+                const uint32_t *q = reinterpret_cast<const uint32_t *>(p - sh / 8);
+                const uint32_t a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2), a3 = sh ? __ldg(q + 3) : 0u;
+                w[r][0] = __funnelshift_r(a0, a1, sh);
+                w[r][1] = __funnelshift_r(a1, a2, sh);
+                w[r][2] = __funnelshift_r(a2, a3, sh);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    w[r][i] = 0;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (4 * i + j < 3 * nc) w[r][i] |= (uint32_t)__ldg(p + 4 * i + j) << (8 * j);
+                }
+            }
+            wh[r] = 0;
+            if (lane == 0 && c > 0)
+                wh[r] = (uint32_t)__ldg(p - 3) << 8 | (uint32_t)__ldg(p - 2) << 16 | (uint32_t)__ldg(p - 1) << 24;
+        }
     }
     // horizontal 3-sums of row r at full-res columns 4c and 4c + 2
     uint32_t hs[kGDR][2];
@@ -129,7 +145,17 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(
         hs[r][0] = __dp4a(g, 0x00000101u, gh);
         hs[r][1] = __dp4a(g, 0x01010100u, 0u);
         const int fy = 8 * band - 1 + r;
-        if (live && !right && r > 0 && fy < H) *reinterpret_cast<uint32_t *>(gf_l + (size_t)fy * W + 4 * c) = g;
+        if (live && !right && r > 0 && fy < H) {
+            uint8_t *o = gf + (size_t)fy * W + 4 * c;
+            if (kAligned) {
+                *reinterpret_cast<uint32_t *>(o) = g;
+            } else if (W % 2 == 0) {                   // (the grey planes start on 256 bytes)
+                *reinterpret_cast<uint16_t *>(o) = (uint16_t)g;
+                if (nc == 4) *reinterpret_cast<uint16_t *>(o + 2) = (uint16_t)(g >> 16);
+            } else {
+                for (int i = 0; i < nc; ++i) o[i] = (uint8_t)(g >> (8 * i));
+            }
+        }
     }
     if (!live) return;
 #pragma unroll
@@ -138,8 +164,14 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(
         if (y >= Y) break;
         const uint32_t m0 = (hs[2 * i][0] + hs[2 * i + 1][0] + hs[2 * i + 2][0] + 4u) / 9u;
         const uint32_t m1 = (hs[2 * i][1] + hs[2 * i + 1][1] + hs[2 * i + 2][1] + 4u) / 9u;
-        // X is even: output pixel 2c starts a 2-byte aligned pair
-        *reinterpret_cast<uint16_t *>(s + (size_t)y * X + 2 * c) = (uint16_t)(m0 | m1 << 8);
+        uint8_t *o = s + (size_t)y * X + 2 * c;
+        if (kAligned || (X % 2 == 0 && 2 * c + 1 < X)) {
+            // X even: output pixel 2c starts a 2-byte aligned pair
+            *reinterpret_cast<uint16_t *>(o) = (uint16_t)(m0 | m1 << 8);
+        } else {
+            if (2 * c < X) o[0] = (uint8_t)m0;
+            if (2 * c + 1 < X) o[1] = (uint8_t)m1;
+        }
     }
 }
 
@@ -399,34 +431,48 @@ cudaError_t launch_grey(const uint8_t *rgb_l, const uint8_t *rgb_r, uint8_t *g_l
     return cudaGetLastError();
 }
 
-cudaError_t launch_downscale(const uint8_t *g_l, const uint8_t *g_r, uint8_t *s_l, uint8_t *s_r,
-                             int W, int H, cudaStream_t s)
+namespace {
+
+template <bool kAligned, int N>
+cudaError_t grey_down_run(const GreyJob *jobs, int n, cudaStream_t s)
 {
-    int X = W / 2, Y = H / 2;
-    dim3 grid((X + 127) / 128, Y, 2);
-    downscale_kernel<<<grid, 128, 0, s>>>(g_l, g_r, s_l, s_r, W, H);
-    return cudaGetLastError();
+    GreyArgs<N> A;
+    A.n = 2 * n;
+    A.start[0] = 0;
+    for (int i = 0; i < n; ++i) {
+        A.job[i] = jobs[i];
+        const int W = jobs[i].W, H = jobs[i].H;
+        const int blocks = ((W + 3) / 4 * (((H + 1) / 2 + kGDB - 1) / kGDB) + kGDT - 1) / kGDT;
+        A.start[2 * i + 1] = A.start[2 * i] + blocks;
+        A.start[2 * i + 2] = A.start[2 * i + 1] + blocks;
+    }
+    return launch_dependent(grey_down_kernel<kAligned, N>, dim3(A.start[2 * n]), dim3(kGDT), 0, s, A);
 }
 
-cudaError_t launch_grey_down(const uint8_t *rgb_l, const uint8_t *rgb_r, uint8_t *gf_l, uint8_t *gf_r,
-                            uint8_t *s_l, uint8_t *s_r, int W, int H, cudaStream_t s, int *launches)
+}  // namespace
+
+cudaError_t launch_grey_down(const GreyJob *jobs, int n, cudaStream_t s, int *launches)
 {
-    const int X = W / 2, Y = H / 2;
-    if (X < 1 || Y < 1) return cudaErrorInvalidValue;
-    const bool aligned = ((reinterpret_cast<uintptr_t>(rgb_l) | reinterpret_cast<uintptr_t>(rgb_r) |
-                           reinterpret_cast<uintptr_t>(gf_l)) & 3) == 0;
-    if (W % 4 != 0 || !aligned) {
-        // rows not word-aligned: the two separate passes
-        *launches += 2;
-        cudaError_t e = launch_grey(rgb_l, rgb_r, gf_l, gf_r, W, H, s);
-        return e != cudaSuccess ? e : launch_downscale(gf_l, gf_r, s_l, s_r, W, H, s);
+    if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
+    GreyJob kind[2][kMaxBatch];
+    int m[2] = {0, 0};
+    for (int i = 0; i < n; ++i) {
+        const GreyJob &j = jobs[i];
+        if (j.W < 2 || j.H < 2) return cudaErrorInvalidValue;
+        const uintptr_t a = reinterpret_cast<uintptr_t>(j.rgb_l) | reinterpret_cast<uintptr_t>(j.rgb_r);
+        const int k = j.W % 4 == 0 && (a & 3) == 0;
+        kind[k][m[k]++] = j;
     }
-    // W a multiple of 4: a thread's group of four lies inside the row
-    const int ncol = W / 4, nband = ((H + 1) / 2 + kGDB - 1) / kGDB;
-    const long nthr = (long)ncol * nband;
-    dim3 grid((unsigned)((nthr + kGDT - 1) / kGDT), 2);
-    *launches += 1;
-    return launch_dependent(grey_down_kernel, grid, dim3(kGDT), 0, s, rgb_l, rgb_r, gf_l, s_l, s_r, W, H, ncol, nband);
+    cudaError_t e = cudaSuccess;
+    if (m[1]) {
+        ++*launches;
+        e = m[1] == 1 ? grey_down_run<true, 2>(kind[1], 1, s) : grey_down_run<true, 2 * kMaxBatch>(kind[1], m[1], s);
+    }
+    if (m[0] && e == cudaSuccess) {
+        ++*launches;
+        e = m[0] == 1 ? grey_down_run<false, 2>(kind[0], 1, s) : grey_down_run<false, 2 * kMaxBatch>(kind[0], m[0], s);
+    }
+    return e;
 }
 
 namespace {

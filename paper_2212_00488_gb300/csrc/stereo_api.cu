@@ -243,9 +243,10 @@ cudaError_t run_stage(stereo_ctx *c, int stage, cudaStream_t s)
     const bool ds = c->p.downscale != 0;
     switch (stage) {
     case STEREO_STAGE_SCALEDOWN: {
-        if (ds)
-            return launch_grey_down(c->in_l, c->in_r, c->gf[0], c->gf[1], c->gs[0], c->gs[1], c->W, c->H, s,
-                                    &c->launches);
+        if (ds) {
+            const GreyJob j{c->in_l, c->in_r, c->gf[0], c->gs[0], c->gs[1], c->W, c->H};
+            return launch_grey_down(&j, 1, s, &c->launches);
+        }
         c->launches++;
         return launch_grey(c->in_l, c->in_r, c->gf[0], c->gf[1], c->W, c->H, s);
     }
@@ -284,11 +285,11 @@ cudaError_t run_stage(stereo_ctx *c, int stage, cudaStream_t s)
     }
     case STEREO_STAGE_REFINE:
         c->launches++;
-        if (ds)   // the scale-up runs in the same kernel
-            return launch_refine_up(c->key[0], c->key[1], c->gs[0], c->gf[0], c->X, c->Y, c->W, c->H, c->p.t_fill,
-                                    c->p.fill_mode, c->out_dl, c->out_dr, c->out_gcp, c->dm, c->dplus, c->out_disp, s);
-        return launch_refine(c->key[0], c->key[1], c->gs[0], c->X, c->Y, c->p.t_fill, c->p.fill_mode, c->out_dl, c->out_dr,
-                             c->out_gcp, c->dm, c->dplus, s);
+        {
+            const RefineJob j{c->key[0], c->key[1], c->gs[0],   c->gf[0],   c->X,  c->Y,     c->W,        c->H,
+                              c->out_dl, c->out_dr, c->out_gcp, c->dm, c->dplus, c->out_disp, 0};
+            return launch_refine(&j, 1, ds, c->p.t_fill, c->p.fill_mode, s);   // ds: with the scale-up
+        }
     case STEREO_STAGE_UPSCALE:
         return cudaSuccess;   // inside the refine stage's kernel (downscaling) or nothing to do
     default:
@@ -689,26 +690,33 @@ CostAggArgs frame_args(const stereo_ctx *c, const FrameWs &f)
     return a;
 }
 
-// Grey, downscale and supports of every frame of a batch: one support launch
-// for all of them.
+// Batches up to this size launch their kernels directly: capturing them as a
+// graph and updating the last one in place takes host time that a batch in a row
+// of batches hides and a lone small one does not (two VGA pairs: 85 us alone
+// through the graph, 72 directly; 58 in a row either way).
+constexpr int kDirectBatch = 4;
+
+// Grey, downscale and supports of every frame of a batch, each step one launch for
+// all of them (without downscaling the grey is one per frame).
 cudaError_t batch_prep(stereo_ctx *c, const std::vector<const stereo_job *> &jobs, const std::vector<FrameWs> &fw,
                        cudaStream_t s, int &launches)
 {
     cudaError_t e = cudaSuccess;
     SupImage im[2 * kMaxBatch];
+    GreyJob gj[kMaxBatch];
     const int n = (int)fw.size();
     for (int k = 0; k < n && e == cudaSuccess; ++k) {
         const stereo_job &j = *jobs[k];
         const FrameWs &f = fw[k];
-        if (c->p.downscale) {
-            e = launch_grey_down(j.left_rgb, j.right_rgb, f.gf[0], f.gf[1], f.gs[0], f.gs[1], f.W, f.H, s, &launches);
-        } else {
+        gj[k] = GreyJob{j.left_rgb, j.right_rgb, f.gf[0], f.gs[0], f.gs[1], f.W, f.H};
+        if (!c->p.downscale) {
             e = launch_grey(j.left_rgb, j.right_rgb, f.gf[0], f.gf[1], f.W, f.H, s);
             launches++;
         }
         for (int i = 0; i < 2; ++i)
             im[2 * k + i] = SupImage{f.gs[i], f.pix[i], f.arm[i], f.armc[i], f.key[i], f.X, f.Y, 0};
     }
+    if (e == cudaSuccess && c->p.downscale) e = launch_grey_down(gj, n, s, &launches);
     if (e == cudaSuccess) {
         e = launch_support(im, 2 * n, c->p.wx, c->p.wy, c->p.tc, c->d_err, s);
         launches++;
@@ -716,14 +724,20 @@ cudaError_t batch_prep(stereo_ctx *c, const std::vector<const stereo_job *> &job
     return e;
 }
 
-cudaError_t batch_post(stereo_ctx *c, const stereo_job &j, const FrameWs &f, cudaStream_t s, int &launches)
+// Cross-check, median, fill and scale-up of every frame of a batch in one launch.
+cudaError_t batch_post(stereo_ctx *c, const std::vector<const stereo_job *> &jobs, const std::vector<FrameWs> &fw,
+                       cudaStream_t s, int &launches)
 {
+    RefineJob rj[kMaxBatch];
+    const int n = (int)fw.size();
+    for (int k = 0; k < n; ++k) {
+        const stereo_job &j = *jobs[k];
+        const FrameWs &f = fw[k];
+        rj[k] = RefineJob{f.key[0], f.key[1], f.gs[0],   f.gf[0], f.X, f.Y, f.W, f.H, j.dl_out, j.dr_out, j.gcp_out, f.dm,
+                          c->p.downscale ? f.dplus : j.disp_out, j.disp_out, 0};
+    }
     launches++;
-    if (c->p.downscale)
-        return launch_refine_up(f.key[0], f.key[1], f.gs[0], f.gf[0], f.X, f.Y, f.W, f.H, c->p.t_fill, c->p.fill_mode,
-                                j.dl_out, j.dr_out, j.gcp_out, f.dm, f.dplus, j.disp_out, s);
-    return launch_refine(f.key[0], f.key[1], f.gs[0], f.X, f.Y, c->p.t_fill, c->p.fill_mode, j.dl_out, j.dr_out,
-                         j.gcp_out, f.dm, j.disp_out, s);
+    return launch_refine(rj, n, c->p.downscale != 0, c->p.t_fill, c->p.fill_mode, s);
 }
 
 std::string batch_signature(const stereo_ctx *c, const std::vector<FrameWs> &fw)
@@ -810,6 +824,11 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
     cudaStream_t us = stream ? (cudaStream_t)stream : c->stream;
     cudaStream_t s = c->stream;
     cudaError_t e;
+    // a stream that is being captured is refused: the batch runs on the
+    // context's stream, which the events would draw into the capture
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(us, &cap)) != cudaSuccess) return cuda_fail(c, e, "stream capture");
+    if (cap != cudaStreamCaptureStatusNone) return cuda_fail(c, cudaErrorStreamCaptureUnsupported, "stream capture");
     if (us != s) {
         if ((e = cudaEventRecord(c->ev_in, us)) != cudaSuccess || (e = cudaStreamWaitEvent(s, c->ev_in, 0)) != cudaSuccess)
             return cuda_fail(c, e, "stream ordering");
@@ -859,41 +878,48 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
         }
     }
 
-    // capture the batch as one graph, then update the last graph in place
     launches = 0;
-    if ((e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
-        return cuda_fail(c, e, "stream capture");
-    e = batch_prep(c, ordered, fw, s, launches);
-    if (e == cudaSuccess) {
-        e = launch_costagg_batch(b, tile, c->num_sms, s);
-        launches++;
-    }
-    for (int k = 0; k < n && e == cudaSuccess; ++k) e = batch_post(c, jobs[order[k]], fw[k], s, launches);
-    cudaGraph_t graph = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(s, &graph);
-    if (e != cudaSuccess || e2 != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
-        cudaGetLastError();
-        return cuda_fail(c, e != cudaSuccess ? e : e2, "batch capture");
-    }
-    // batches of one size share the graph topology, so the last graph of that
-    // size is updated in place; a new size or tile shape instantiates anew
-    cudaGraphExec_t &exec = c->bexec[n];
-    if (exec) {
-        cudaGraphExecUpdateResultInfo info;
-        if (cudaGraphExecUpdate(exec, graph, &info) != cudaSuccess) {
-            cudaGetLastError();
-            cudaGraphExecDestroy(exec);
-            exec = nullptr;
+    auto run = [&]() -> cudaError_t {
+        cudaError_t r = batch_prep(c, ordered, fw, s, launches);
+        if (r == cudaSuccess) {
+            r = launch_costagg_batch(b, tile, c->num_sms, s);
+            launches++;
         }
-    }
-    if (!exec && (e = cudaGraphInstantiate(&exec, graph, 0)) != cudaSuccess) {
+        return r == cudaSuccess ? batch_post(c, ordered, fw, s, launches) : r;
+    };
+    if (n <= kDirectBatch) {
+        if ((e = run()) != cudaSuccess) return cuda_fail(c, e, "kernel launch");
+    } else {
+        // capture the batch as one graph, then update the last graph in place
+        if ((e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
+            return cuda_fail(c, e, "stream capture");
+        e = run();
+        cudaGraph_t graph = nullptr;
+        cudaError_t e2 = cudaStreamEndCapture(s, &graph);
+        if (e != cudaSuccess || e2 != cudaSuccess) {
+            if (graph) cudaGraphDestroy(graph);
+            cudaGetLastError();
+            return cuda_fail(c, e != cudaSuccess ? e : e2, "batch capture");
+        }
+        // batches of one size share the graph topology, so the last graph of that
+        // size is updated in place; a new size or tile shape instantiates anew
+        cudaGraphExec_t &exec = c->bexec[n];
+        if (exec) {
+            cudaGraphExecUpdateResultInfo info;
+            if (cudaGraphExecUpdate(exec, graph, &info) != cudaSuccess) {
+                cudaGetLastError();
+                cudaGraphExecDestroy(exec);
+                exec = nullptr;
+            }
+        }
+        if (!exec && (e = cudaGraphInstantiate(&exec, graph, 0)) != cudaSuccess) {
+            cudaGraphDestroy(graph);
+            exec = nullptr;
+            return cuda_fail(c, e, "graph instantiate");
+        }
         cudaGraphDestroy(graph);
-        exec = nullptr;
-        return cuda_fail(c, e, "graph instantiate");
+        if ((e = cudaGraphLaunch(exec, s)) != cudaSuccess) return cuda_fail(c, e, "graph launch");
     }
-    cudaGraphDestroy(graph);
-    if ((e = cudaGraphLaunch(exec, s)) != cudaSuccess) return cuda_fail(c, e, "graph launch");
     if (us != s) {
         if ((e = cudaEventRecord(c->ev_out, s)) != cudaSuccess || (e = cudaStreamWaitEvent(us, c->ev_out, 0)) != cudaSuccess)
             return cuda_fail(c, e, "stream ordering");
