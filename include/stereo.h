@@ -199,7 +199,9 @@ STEREO_API int stereo_last_launch_count(const stereo_ctx *ctx);
  * 16-bit for wx up to 28, 6: 48x8 32-bit (slabs of 8 disparities, two threads
  * per column), 7: 64x4 32-bit for wx up to 174 with 8 producer warps (the wide
  * windows of Table I, up to the library's limit of 141), 8: 88x4 32-bit for
- * wx up to 66 with 8 producer warps. A frame whose tiles leave SMs idle is cut
+ * wx up to 66 with 8 producer warps. Shapes 3 and 8 take packed 16-bit prefixes
+ * (96 and 88 columns) where (wx+1) times the largest matching cost stays below
+ * 2^16. A frame whose tiles leave SMs idle is cut
  * into bands of rows, each with its own tiles.
  * 16-bit row prefixes need max(2*wx+1, 7) times the largest matching cost
  * below 2^16. Every shape gives the same result; they differ only in speed.

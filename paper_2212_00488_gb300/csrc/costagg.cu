@@ -142,7 +142,8 @@ constexpr Roles producer_roles(int ncw, int npw)
     }
     return r;
 }
-template <int XS_, int DS_, int KE_, int RS_, bool S16_, int DPT_, int NPW_, int WX_, int NS_>
+template <int XS_, int DS_, int KE_, int RS_, bool S16_, int DPT_, int NPW_, int WX_, int NS_,
+          bool SPLIT_ = false>
 struct Tile {
     static constexpr int XS = XS_;            // columns per base
     static constexpr int DS = DS_;            // disparities per CTA
@@ -150,6 +151,7 @@ struct Tile {
     static constexpr int RS = RS_;            // row slots between producers and consumers
     static constexpr bool S16 = S16_;         // pairs of disparities share a prefix word (window sums < 2^16)
     static constexpr int WX = WX_;            // largest wx the tile takes
+    static constexpr bool SPLIT = SPLIT_;     // 16-bit form with a window's two sides below 2^16 each, not their sum
     static constexpr int NS = NS_;            // time of a row step in ns with every SM busy (estimate())
     static constexpr int DPT = DPT_;          // disparities per consumer thread
     static constexpr int G = DS / DPT;        // consumer threads per column (adjacent lanes)
@@ -469,11 +471,20 @@ __device__ __forceinline__ void costagg_tile(const CostAggArgs &a, const int x0,
         if constexpr (T::S16) {
             const uint2 *w = prow0 + slot * (2 * T::SWP);
             const uint2 h = w[hi], l = w[-lo];
-            const uint32_t w0 = h.x - l.x, w1 = h.y - l.y;
-            cax[0] = __byte_perm(w0, 0u, 0x4104);
-            cax[1] = __byte_perm(w0, 0u, 0x4324);
-            cax[2] = __byte_perm(w1, 0u, 0x4104);
-            cax[3] = __byte_perm(w1, 0u, 0x4324);
+            auto place = [&](uint32_t w0, uint32_t w1, int k) {
+                return __byte_perm(k < 2 ? w0 : w1, 0u, k % 2 ? 0x4324 : 0x4104);
+            };
+            if constexpr (T::SPLIT) {
+                // the window in two, at the pixel's own column
+                const uint2 m = w[0];
+                const uint32_t a0 = h.x - m.x, a1 = h.y - m.y, b0 = m.x - l.x, b1 = m.y - l.y;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cax[k] = place(a0, a1, k) + place(b0, b1, k);
+            } else {
+                const uint32_t w0 = h.x - l.x, w1 = h.y - l.y;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cax[k] = place(w0, w1, k);
+            }
         } else {
             const uint32_t *r0 = srow0 + slot * (T::DS * T::SWP);
 #pragma unroll
@@ -684,14 +695,28 @@ using T6 = Tile<48, 8, 5, 4, false, 4, 4, 52, 259>;
 using T7 = Tile<64, 4, 13, 8, false, 4, 8, 174, 180>;
 // wx up to 66 (Table I's W_x = 61) with 32-bit prefixes: 7 prefix entries
 // per producer lane leave room for 8 producer warps and row slots
-using T8 = Tile<88, 4, 7, 8, false, 4, 8, 66, 153>;
+using T8 = Tile<88, 4, 7, 8, false, 4, 8, 66, 163>;
+
+// Tiles 3 and 8 where the sums of a window's two sides stay below 2^16 though
+// their total need not (W_x 41 and 61 at cost scale 512): packed prefixes after
+// all, with one more load per window. Faster than four 32-bit prefixes a row
+// (1436 x 992, W_x 41: 134 -> 94 us, W_x 61: 160 -> 140 us).
+using T3S = Tile<96, 4, 7, 8, true, 4, 8, 58, 166, true>;
+using T8S = Tile<88, 4, 7, 12, true, 4, 12, 66, 140, true>;
+bool split_fits(const CostAggArgs &a)
+{
+    return (uint64_t)std::max(a.wx + 1, T3S::KE) * a.P < 65536u;
+}
 
 template <class T> struct Tag { using type = T; };
 
-// Calls f(Tag<T>) for the tile shape with the given id; false for an unknown id.
+// Calls f(Tag<T>) for the tile shape with the given id, in its split form where
+// `split`; false for an unknown id.
 template <class F>
-bool with_tile(int id, F &&f)
+bool with_tile(int id, bool split, F &&f)
 {
+    if (split && id == 3) { f(Tag<T3S>{}); return true; }
+    if (split && id == 8) { f(Tag<T8S>{}); return true; }
     switch (id) {
     case 0: f(Tag<T0>{}); return true;
     case 1: f(Tag<T1>{}); return true;
@@ -713,7 +738,7 @@ bool fits(const CostAggArgs &a)
     if (a.wx > T::WX) return false;
     // 16-bit prefixes need every horizontal window sum, and every producer
     // lane's sum of KE costs, below 2^16
-    return !T::S16 || (uint64_t)max(2 * a.wx + 1, T::KE) * a.P < 65536u;
+    return !T::S16 || (uint64_t)max(T::SPLIT ? a.wx + 1 : 2 * a.wx + 1, T::KE) * a.P < 65536u;
 }
 
 
@@ -815,7 +840,8 @@ cudaError_t costagg_setup()
 {
     cudaError_t e = cudaSuccess;
     for (int id = 0; id < kNumTiles && e == cudaSuccess; ++id)
-        with_tile(id, [&](auto tag) { e = setup_one<typename decltype(tag)::type>(); });
+        for (bool split : {false, true})
+            if (e == cudaSuccess) with_tile(id, split, [&](auto tag) { e = setup_one<typename decltype(tag)::type>(); });
     return e;
 }
 
@@ -824,7 +850,7 @@ int costagg_pick(const CostAggArgs &a, int nsm)
     int best = -1;
     double bt = 0;
     for (int id = 0; id < kNumTiles; ++id)
-        with_tile(id, [&](auto tag) {
+        with_tile(id, split_fits(a), [&](auto tag) {
             using T = typename decltype(tag)::type;
             if (!fits<T>(a)) return;
             int band;
@@ -840,7 +866,7 @@ int costagg_pick(const CostAggArgs &a, int nsm)
 bool costagg_fits(const CostAggArgs &a, int tile)
 {
     bool ok = false;
-    with_tile(tile, [&](auto tag) { ok = fits<typename decltype(tag)::type>(a); });
+    with_tile(tile, split_fits(a), [&](auto tag) { ok = fits<typename decltype(tag)::type>(a); });
     return ok;
 }
 
@@ -848,7 +874,8 @@ cudaError_t launch_costagg_batch(BatchArgs &b, int tile, int nsm, cudaStream_t s
 {
     if (b.njobs < 1 || b.njobs > kMaxBatch) return cudaErrorInvalidValue;
     cudaError_t e = cudaErrorInvalidValue;
-    with_tile(tile, [&](auto tag) { e = launch_batch_one<typename decltype(tag)::type>(b, nsm, s); });
+    with_tile(tile, split_fits(b.job[0]),
+              [&](auto tag) { e = launch_batch_one<typename decltype(tag)::type>(b, nsm, s); });
     return e;
 }
 
@@ -857,7 +884,7 @@ cudaError_t launch_costagg(const CostAggArgs &a, cudaStream_t s)
     if (a.wy > kMaxWy || a.wy < 0 || a.wx < 0 || a.wx > kMaxWx) return cudaErrorInvalidValue;
     const int tile = a.tile >= 0 ? a.tile : costagg_pick(a, a.num_sms);
     cudaError_t e = cudaErrorInvalidValue;
-    with_tile(tile, [&](auto tag) {
+    with_tile(tile, split_fits(a), [&](auto tag) {
         using T = typename decltype(tag)::type;
         if (fits<T>(a)) e = launch_one<T>(a, s);
     });

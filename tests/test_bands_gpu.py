@@ -25,16 +25,30 @@ def _built():
 @pytest.mark.parametrize("tile", [-1, 0, 3, 4, 5, 8])
 @pytest.mark.parametrize("W,H,D", [(40, 901, 9), (95, 130, 3), (96, 61, 4), (97, 300, 5), (193, 257, 75)])
 def test_bands_and_overlapping_slabs(W, H, D, tile):
+    _check(W, H, D, tile)
+
+
+# windows above 2^16 that the split form of tiles 3 and 8 takes (wx 41 and 61 at
+# scale 512, and at the last scale it takes), and the 32-bit form just past it
+@pytest.mark.parametrize("tile,wx,scale", [(3, 41, 512), (8, 61, 512), (-1, 58, 512), (3, 58, 587), (3, 58, 588),
+                                           (8, 66, 517), (8, 66, 518), (-1, 41, 1300)])
+def test_windows_above_16_bits(tile, wx, scale):
+    _check(300, 90, 18, tile, wx=wx, wy=15, cost_scale=scale)
+
+
+def _check(W, H, D, tile, **params):
     from paper_2212_00488_gb300 import Stereo, _lib
     s = scenes.make_scene(W, H, D, planes=5, seed=W + H)
     left, right = s.left // 64 + 100, s.right // 64 + 100          # arms at their caps
-    st = Stereo(0, downscale=0)
+    st = Stereo(0, downscale=0, **params)
     _lib.stereo_set_tile(st.ctx, tile)
     out = st(torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda(), D, maps=True)
     torch.cuda.synchronize()
     st.close()
     p = oracle.Params()
     p.downscale = 0
+    for k, v in params.items():
+        setattr(p, k, v)
     ref = oracle.pipeline(left, right, D, p)
     for k in ("dl", "dr", "gcp", "disp"):
         got, want = getattr(out, k).cpu().numpy(), getattr(ref, k)
