@@ -188,10 +188,11 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__
 // hides the latency of each, and a warp stops when none of its 512 arms goes
 // on (tested every four steps). Bound by the ALU pipe. At 718 x 496 (two
 // images) 34.5 us with one thread following each arm eight pixels at a time
-// and a queue for the arms that go on, 18.2 us now (cold L2, both).
+// and a queue for the arms that go on, 16.5 us now (cold L2, both).
 constexpr int kSX = 128, kSY = 16;           // pixels of a CTA
 constexpr int kSupNT = 512;                  // 4 directions x 4 row quads
 constexpr int kSupWarps = kSupNT / 32;
+constexpr int kSupStage = 5;                 // staged column words per thread and pass
 static_assert(kSupWarps == 4 * (kSY / 4) && kSupWarps == kSY, "a warp per (direction, quad), and per census row");
 constexpr uint32_t kHi = 0x80808080u;
 
@@ -207,23 +208,57 @@ __host__ __device__ constexpr int sup_smem(int wx, int wy)
 }
 static_assert(sup_smem(kMaxWx, kMaxWy) <= 48 * 1024, "fits the default shared memory of a CTA");
 
-// Four pixels x .. x + 3 of row `row` (columns clamped to the image). The
-// pixels come from the aligned words that hold them: a word that starts in the
-// image ends inside its allocation (planes start on 256-byte boundaries of a
-// larger one, or their size is a whole number of words).
+// Four pixels x .. x + 3 of row `row` (columns clamped to the image; x is a
+// multiple of 4). The pixels come from the aligned words that hold them: a word
+// that starts in the image ends inside its allocation (planes start on 256-byte
+// boundaries of a larger one, or their size is a whole number of words). No
+// branch, so that several loads are in flight: a quad over the right edge is
+// the last whole one, its bytes moved down and its last byte repeated.
+template <bool kNarrow>
 __device__ __forceinline__ uint32_t load_quad(const uint8_t *row, int x, int X)
 {
-    if (x >= 0 && x + 3 < X) {
-        const uintptr_t a = reinterpret_cast<uintptr_t>(row + x);
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(a & ~(uintptr_t)3);
-        const uint32_t sh = (uint32_t)(a & 3) * 8;
-        const uint32_t w0 = __ldg(w);
-        return sh ? __funnelshift_r(w0, __ldg(w + 1), sh) : w0;
-    }
-    uint32_t v = 0;
+    if (kNarrow) {                                         // fewer than four columns
+        uint32_t v = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v |= (uint32_t)__ldg(row + min(max(x + i, 0), X - 1)) << (8 * i);
-    return v;
+        for (int i = 0; i < 4; ++i) v |= (uint32_t)__ldg(row + min(max(x + i, 0), X - 1)) << (8 * i);
+        return v;
+    }
+    const int xc = min(max(x, 0), X - 4);
+    const uintptr_t a = reinterpret_cast<uintptr_t>(row + xc);
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(a & ~(uintptr_t)3);
+    const uint32_t sh = (uint32_t)(a & 3) * 8;
+    const uint32_t q = __funnelshift_r(__ldg(w), __ldg(w + (sh != 0)), sh);
+    return __byte_perm(q, 0u, x < 0 ? 0u : 0x33333210u >> (4 * min(x - xc, 4)));
+}
+
+// Stages the rows of the horizontal scans and the columns of the vertical ones,
+// the loads of one pass (a 21 x 31 window takes one) before its first store.
+template <bool kNarrow>
+__device__ __forceinline__ void stage(const SupImage &I, uint32_t *rows, uint32_t *cols, int x0, int y0, int hw, int wy)
+{
+    constexpr int P = kSX / 4, B = kSupStage;
+    const int X = I.X, Y = I.Y, RW = P + 2 * hw, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i0 = threadIdx.x; i0 < (kSY + 2) * RW; i0 += 2 * kSupNT) {
+        uint32_t v[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = min(i0 + k * kSupNT, (kSY + 2) * RW - 1), r = i / RW;
+            v[k] = load_quad<kNarrow>(I.g + (size_t)min(max(y0 - 1 + r, 0), Y - 1) * X, x0 + 4 * (i - r * RW - hw), X);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (i0 + k * kSupNT < (kSY + 2) * RW) rows[i0 + k * kSupNT] = v[k];
+    }
+    if (!I.arm) return;
+    for (int r = warp; r < kSY + 2 * wy; r += B * kSupWarps) {
+        uint32_t v[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k)
+            v[k] = load_quad<kNarrow>(I.g + (size_t)min(max(y0 - wy + r + k * kSupWarps, 0), Y - 1) * X, x0 + 4 * lane, X);
+#pragma unroll
+        for (int k = 0; k < B; ++k)
+            if (r + k * kSupWarps < kSY + 2 * wy) cols[(r + k * kSupWarps) * P + lane] = v[k];
+    }
 }
 
 // Byte compare of a scan step: bit 7 of each byte of the result is set when
@@ -310,8 +345,8 @@ struct SupArgs {
     SupImage im[N];
 };
 
-template <int N, bool kBig>
-__global__ void __launch_bounds__(kSupNT, 3) support_kernel(const __grid_constant__ SupArgs<N> A)
+template <int N, bool kBig, int kPerSM>
+__global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_constant__ SupArgs<N> A)
 {
     extern __shared__ __align__(16) uint32_t sup[];
     pdl_trigger();
@@ -330,13 +365,10 @@ __global__ void __launch_bounds__(kSupNT, 3) support_kernel(const __grid_constan
     pdl_wait();                                            // the grey image of the previous kernel
     if ((blockIdx.x | threadIdx.x) == 0) *A.err = 0u;
 
-    for (int i = threadIdx.x; i < (kSY + 2) * RW; i += kSupNT) {
-        const int r = i / RW, w = i - r * RW;
-        rows[i] = load_quad(I.g + (size_t)min(max(y0 - 1 + r, 0), Y - 1) * X, x0 + 4 * (w - hw), X);
-    }
-    if (I.arm)
-        for (int r = warp; r < kSY + 2 * wy; r += kSupWarps)
-            cols[r * P + lane] = load_quad(I.g + (size_t)min(max(y0 - wy + r, 0), Y - 1) * X, x0 + 4 * lane, X);
+    if (X >= 4)
+        stage<false>(I, rows, cols, x0, y0, hw, wy);
+    else
+        stage<true>(I, rows, cols, x0, y0, hw, wy);
     __syncthreads();
 
     if (I.arm) {
@@ -492,9 +524,21 @@ cudaError_t support_run(const SupImage *im, int n, int wx, int wy, int tc, uint3
         A.im[i].nx = (im[i].X + kSX - 1) / kSX;
         A.start[i + 1] = A.start[i] + A.im[i].nx * ((im[i].Y + kSY - 1) / kSY);
     }
-    const dim3 grid(A.start[n]), block(kSupNT);
-    return tc < 128 ? launch_dependent(support_kernel<N, false>, grid, block, sup_smem(wx, wy), s, A)
-                    : launch_dependent(support_kernel<N, true>, grid, block, sup_smem(wx, wy), s, A);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const auto go = [&](auto kernel) {
+        return launch_dependent(kernel, dim3(A.start[n]), dim3(kSupNT), sup_smem(wx, wy), s, A);
+    };
+    // Images whose CTAs all run at once with two on an SM take the form with 64
+    // registers, which has more scan steps' loads in flight; more CTAs take
+    // three on an SM (40 registers). 360 x 248: 15.9 -> 11.4 us, 640 x 480 (300
+    // CTAs): 14.7 -> 11.4 us; at 372 and 544 CTAs there is nothing to choose,
+    // from 2040 (3840 x 2160, halved) three are the faster, 66.7 against 64.4 us.
+    if (A.start[n] <= 2 * sms)
+        return tc < 128 ? go(support_kernel<N, false, 2>) : go(support_kernel<N, true, 2>);
+    return tc < 128 ? go(support_kernel<N, false, 3>) : go(support_kernel<N, true, 3>);
 }
 
 }  // namespace

@@ -1,7 +1,7 @@
 """The support kernel (mini-census codes and cross arms) against the oracle,
 integer for integer, at the edges of its 128 x 16 pixel tiles, of its four-pixel
 words and of its byte compare (tc on both sides of 128), with arms of every
-length up to the caps."""
+length up to the caps, with few CTAs (two on an SM) and with more (three)."""
 import numpy as np
 import pytest
 
@@ -20,7 +20,8 @@ def _built():
     build.build()
 
 
-@pytest.mark.parametrize("W,H", [(1, 1), (5, 3), (127, 15), (128, 16), (129, 17), (390, 70)])
+@pytest.mark.parametrize("W,H", [(1, 1), (3, 9), (4, 5), (5, 3), (127, 15), (128, 16), (129, 17), (390, 70),
+                                 (1217, 255)])
 @pytest.mark.parametrize("tc,wx,wy", [(0, 21, 31), (13, 1, 1), (13, 6, 30), (127, 21, 31), (128, 21, 31),
                                       (255, 141, 31), (256, 5, 3)])
 def test_codes_and_arms_at_tile_edges(W, H, tc, wx, wy):
