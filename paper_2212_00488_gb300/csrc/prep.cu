@@ -66,7 +66,7 @@ __global__ void grey_kernel(const uint8_t *__restrict__ rgb_l, const uint8_t *__
 // kAligned: W a multiple of 4 and word-aligned rows. Else a row's words are funnel
 // shifts of the aligned words that hold its pixels, the last group of a row may
 // be partial, and stores go by halfwords or bytes (1482 x 994: 10.3 us as two
-// kernels, 8.8 now). The frames of a batch share a launch of each kind.
+// kernels, 8.8 as one with a branch a row, 5.8 now). The frames of a batch share a launch of each kind.
 constexpr int kGDT = 128;                  // threads per CTA
 constexpr int kGDB = 4;                    // output rows per thread
 constexpr int kGDR = 2 * kGDB + 1;         // full-res rows per thread
@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__
     const uint8_t *rgb = right ? J.rgb_r : J.rgb_l;
     uint8_t *s = right ? J.s_r : J.s_l, *gf = J.gf_l;
     const int nc = min(4, W - 4 * c);                 // columns of the group
+    const uint8_t *end = rgb + (size_t)W * H * 3;
     pdl_wait();   // launched early behind the previous frame's last kernel, which still reads gf and s
     uint32_t w[kGDR][3], wh[kGDR];
 #pragma unroll
@@ -110,26 +111,36 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__
             for (int i = 0; i < 3; ++i) w[r][i] = __ldg(q + i);
             wh[r] = lane == 0 && c > 0 ? __ldg(q - 1) : 0u;
         } else {
-            // whole groups whose last word ends inside the image's bytes
+            // Sixteen aligned bytes hold the group's twelve; a partial group takes
+            // bytes of the next row along, which no result of the image uses.
             const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3) * 8;
-            if (nc == 4 && (fy + 1 < H || 4 * c + 8 <= W)) {
-                const uint32_t *q = reinterpret_cast<const uint32_t *>(p - sh / 8);
-                const uint32_t a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2), a3 = sh ? __ldg(q + 3) : 0u;
-                w[r][0] = __funnelshift_r(a0, a1, sh);
-                w[r][1] = __funnelshift_r(a1, a2, sh);
-                w[r][2] = __funnelshift_r(a2, a3, sh);
-            } else {
+            const uint32_t *q = reinterpret_cast<const uint32_t *>(p - sh / 8);
+            uint32_t a[4] = {0, 0, 0, 0}, h = 0;
+            if (reinterpret_cast<const uint8_t *>(q + 4) <= end) {
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    w[r][i] = 0;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (4 * i + j < 3 * nc) w[r][i] |= (uint32_t)__ldg(p + 4 * i + j) << (8 * j);
-                }
+                for (int i = 0; i < 4; ++i) a[i] = __ldg(q + i);
+                if (lane == 0 && c > 0) h = __ldg(q - 1);
             }
-            wh[r] = 0;
-            if (lane == 0 && c > 0)
-                wh[r] = (uint32_t)__ldg(p - 3) << 8 | (uint32_t)__ldg(p - 2) << 16 | (uint32_t)__ldg(p - 1) << 24;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) w[r][i] = __funnelshift_r(a[i], a[i + 1], sh);
+            wh[r] = __funnelshift_r(h, a[0], sh);
+        }
+    }
+    if (!kAligned && 8 * band + kGDR - 2 >= H - 3) {
+        // groups whose sixteen bytes would end past the image (in its last three
+        // rows): byte loads, once for a row that is taken more than once
+#pragma unroll 1
+        for (int f = max(H - 3, 0); f < H; ++f) {
+            const uint8_t *p = rgb + ((size_t)f * W + 4 * c) * 3;
+            if (p - (reinterpret_cast<uintptr_t>(p) & 3) + 16 <= end) continue;
+            uint32_t v[3] = {0, 0, 0}, h = 0;
+#pragma unroll
+            for (int j = 0; j < 12; ++j)
+                if (j < 3 * nc) v[j >> 2] |= (uint32_t)__ldg(p + j) << (8 * (j & 3));
+            if (c > 0) h = (uint32_t)__ldg(p - 3) << 8 | (uint32_t)__ldg(p - 2) << 16 | (uint32_t)__ldg(p - 1) << 24;
+#pragma unroll
+            for (int k = 0; k < kGDR; ++k)
+                if (min(max(8 * band - 1 + k, 0), H - 1) == f) w[k][0] = v[0], w[k][1] = v[1], w[k][2] = v[2], wh[k] = h;
         }
     }
     // horizontal 3-sums of row r at full-res columns 4c and 4c + 2
