@@ -227,11 +227,12 @@ typedef struct {
 } stereo_job;
 
 /* Up to 32 pairs in one call (the batched form of the method; the paper
- * processes one pair at a time). Preparation and post-processing run per
- * frame, the fused cost + aggregation + WTA of all frames runs as one
- * persistent kernel taking (frame, strip, slab) tiles largest frame first;
- * the whole batch is one CUDA graph, re-captured and updated in place on each
- * call (batches of up to four frames are launched directly). Each frame's maps equal stereo_compute's for that frame exactly.
+ * processes one pair at a time). Preparation and post-processing take one
+ * launch a step for all frames, the fused cost + aggregation + WTA of all
+ * frames runs as one persistent kernel taking (frame, strip, slab) tiles
+ * largest frame first; a batch of more than four frames is one CUDA graph,
+ * re-captured and updated in place on each call, a smaller one is launched
+ * directly. Each frame's maps equal stereo_compute's for that frame exactly.
  * With the automatic tile (stereo_set_tile(-1)) the first batch of a given
  * signature (frame shapes, parameters, GPU) times every tile shape that fits
  * and remembers the fastest; stereo_tune_save / stereo_tune_load keep those
