@@ -16,8 +16,8 @@
 //    land inside [x0+sft-wx, x0+sft+XS+DS-1+wx), next to the left windows. The
 //    shift back by sft uses up the spare entries of the prefix rows, so that at
 //    718 columns 96 of them give every slab 8 strips, 152 CTAs in all.
-//  * Output rows: a band of the frame, the whole of it where the tiles fill the
-//    GPU. The sweep starts wy rows above the band and ends wy below.
+//  * Output rows: all of them in the tiles that fill whole waves of the GPU, a band
+//    in the rest. The sweep starts wy rows above the band and ends wy below.
 //
 // What bounds it: the instructions of the few warps an SM has room for beside
 // the ring (issue slots 60-70 % used, shared-memory pipe 75 %). 718 x 496 x 73:
@@ -628,19 +628,25 @@ __host__ __device__ __forceinline__ int tiles_of(const CostAggArgs &a)
     return n;
 }
 
-// Tile t of a frame cut into row bands of a.band rows: all strips and slabs of
-// the first band, then of the next.
+// CTA t of a frame: the first a.head tiles (strip, slab) are swept from the first
+// row to the last, the others in row bands of a.band rows: all of them in the
+// first band, then in the next.
 template <class T>
 __device__ __forceinline__ void run_tile(const CostAggArgs &a, int t, unsigned char *smem, bool reuse)
 {
-    int band = 0;
-    for (const int n = tiles_of<T>(a); t >= n; t -= n) ++band;
+    int ya = 0, yb = a.Y;
+    if (t >= a.head) {
+        const int rest = tiles_of<T>(a) - a.head, band = (t - a.head) / rest;
+        t -= band * rest;
+        ya = band * a.band;
+        yb = min(ya + a.band, a.Y);
+    }
     int s = 0;
     for (int n = slab_strips<T>(a, 0); t >= n; n = slab_strips<T>(a, s)) {
         t -= n;
         ++s;
     }
-    costagg_tile<T>(a, t * T::XS, slab_d0<T>(a, s), band * a.band, min((band + 1) * a.band, a.Y), smem, reuse);
+    costagg_tile<T>(a, t * T::XS, slab_d0<T>(a, s), ya, yb, smem, reuse);
 }
 
 template <class T>
@@ -795,6 +801,7 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
     for (int j = 0; j < b.njobs; ++j) {
         CostAggArgs &a = b.job[j];
         a.band = band_rows(a, nb);
+        a.head = 0;
         b.tile_start[j] = b.total_tiles;
         b.total_tiles += tiles_of<T>(a) * ((a.Y + a.band - 1) / a.band);
     }
@@ -806,21 +813,31 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Time of a frame in ns with this tile in the best cut into bands: waves of
-// CTAs times their row steps times the tile's measured time per step. A small
-// frame's tiles leave SMs idle: 360 x 248 x 36 took 38.1 us in one band (56 CTAs
-// of 152 SMs), 17.8 us cut into bands.
+// Time of a frame in ns with this tile in its best cut, waves of CTAs times their
+// row steps times the tile's measured time per step; sets the cut. A small
+// frame's tiles leave SMs idle: all of them go in bands (360 x 248 x 36: 38.1 us
+// in one band, 56 CTAs of 152 SMs, 17.8 us cut). A larger frame's last wave does:
+// whole waves of tiles stay in one piece, without the wy rows a band sweeps above
+// and below its own, and the rest go in bands (1436 x 992, W_x 61, 171 tiles:
+// all in two bands 140 us, 152 whole and 19 in bands 106; 3840 x 2160, 4.4
+// waves: 707 and 644 us).
 template <class T>
-double estimate(const CostAggArgs &a, int nsm, int &band)
+double estimate(const CostAggArgs &a, int nsm, int &head, int &band)
 {
+    const int tiles = tiles_of<T>(a), waves = tiles / nsm;
     double best = 0;
-    for (int n = 1; n <= kMaxBands; ++n) {
-        const int rows = band_rows(a, n);
-        const long ctas = (long)tiles_of<T>(a) * ((a.Y + rows - 1) / rows);
-        const double t = (double)((ctas + nsm - 1) / nsm) * band_steps(a, rows) * T::NS;
-        if (n == 1 || t < best) {
-            best = t;
-            band = rows;
+    head = -1;
+    for (int k : {0, waves}) {
+        const int rest = tiles - k * nsm;
+        for (int n = 1; n <= kMaxBands; ++n) {
+            const int rows = band_rows(a, n);
+            const long ctas = (long)rest * ((a.Y + rows - 1) / rows);
+            const double t = ((double)k * band_steps(a, a.Y) + (double)((ctas + nsm - 1) / nsm) * band_steps(a, rows)) * T::NS;
+            if (head < 0 || t < best) {
+                best = t;
+                head = k * nsm;
+                band = rows;
+            }
         }
     }
     return best;
@@ -829,8 +846,8 @@ double estimate(const CostAggArgs &a, int nsm, int &band)
 template <class T>
 cudaError_t launch_one(CostAggArgs a, cudaStream_t s)
 {
-    estimate<T>(a, a.num_sms, a.band);
-    const int ctas = tiles_of<T>(a) * ((a.Y + a.band - 1) / a.band);
+    estimate<T>(a, a.num_sms, a.head, a.band);
+    const int ctas = a.head + (tiles_of<T>(a) - a.head) * ((a.Y + a.band - 1) / a.band);
     return launch_dependent(costagg_wta_kernel<T>, dim3(ctas), dim3(T::NT), T::BYTES, s, a);
 }
 
@@ -853,8 +870,8 @@ int costagg_pick(const CostAggArgs &a, int nsm)
         with_tile(id, split_fits(a), [&](auto tag) {
             using T = typename decltype(tag)::type;
             if (!fits<T>(a)) return;
-            int band;
-            const double est = estimate<T>(a, nsm, band);
+            int head, band;
+            const double est = estimate<T>(a, nsm, head, band);
             if (best < 0 || est < bt) {
                 best = id;
                 bt = est;

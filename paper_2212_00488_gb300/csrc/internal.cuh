@@ -55,7 +55,7 @@ struct CostAggArgs {
     uint32_t P;                      // cost of a match outside the image
     int tile;                        // tile shape id, -1 = pick from the shape
     int num_sms;                     // SMs of the device (for the pick)
-    int band;                        // rows of a band (filled by the launcher)
+    int head, band;                  // tiles swept in one piece, rows of the others' bands (filled by the launcher)
 };
 
 // Programmatic dependent launch between the kernels of a frame: a kernel

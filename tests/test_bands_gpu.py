@@ -28,6 +28,12 @@ def test_bands_and_overlapping_slabs(W, H, D, tile):
     _check(W, H, D, tile)
 
 
+# more tiles than one wave: whole tiles first, the rest in bands
+@pytest.mark.parametrize("tile", [-1, 0, 1, 2, 3, 4, 5, 6, 7, 8])
+def test_whole_tiles_and_banded_rest(tile):
+    _check(1000, 130, 75, tile)
+
+
 # windows above 2^16 that the split form of tiles 3 and 8 takes (wx 41 and 61 at
 # scale 512, and at the last scale it takes), and the 32-bit form just past it
 @pytest.mark.parametrize("tile,wx,scale", [(3, 41, 512), (8, 61, 512), (-1, 58, 512), (3, 58, 587), (3, 58, 588),
