@@ -201,8 +201,8 @@ STEREO_API int stereo_last_launch_count(const stereo_ctx *ctx);
  * windows of Table I, up to the library's limit of 141), 8: 88x4 32-bit for
  * wx up to 66 with 8 producer warps. Shapes 3 and 8 take packed 16-bit prefixes
  * (96 and 88 columns) where (wx+1) times the largest matching cost stays below
- * 2^16. A frame whose tiles leave SMs idle is cut
- * into bands of rows, each with its own tiles.
+ * 2^16. Tiles that do not
+ * fill a whole wave of the SMs are cut into bands of rows.
  * 16-bit row prefixes need max(2*wx+1, 7) times the largest matching cost
  * below 2^16. Every shape gives the same result; they differ only in speed.
  * A compute with a shape that does not fit the parameters fails with EINVAL. */
