@@ -701,7 +701,7 @@ using T6 = Tile<48, 8, 5, 4, false, 4, 4, 52, 259>;
 using T7 = Tile<64, 4, 13, 8, false, 4, 8, 174, 180>;
 // wx up to 66 (Table I's W_x = 61) with 32-bit prefixes: 7 prefix entries
 // per producer lane leave room for 8 producer warps and row slots
-using T8 = Tile<88, 4, 7, 8, false, 4, 8, 66, 163>;
+using T8 = Tile<88, 4, 7, 8, false, 4, 8, 66, 170>;
 
 // Tiles 3 and 8 where the sums of a window's two sides stay below 2^16 though
 // their total need not (W_x 41 and 61 at cost scale 512): packed prefixes after
