@@ -690,6 +690,38 @@ CostAggArgs frame_args(const stereo_ctx *c, const FrameWs &f)
     return a;
 }
 
+// A call's work on the context's stream, between the caller's stream before and
+// after it: enter() lets the context's stream wait for the caller's, leave() the
+// caller's for everything queued since. A call that returns early on an error
+// leaves too (destructor): kernels queued before the error still read the
+// caller's buffers.
+class OnOwnStream {
+public:
+    OnOwnStream(stereo_ctx *c, cudaStream_t caller) : c_(c), caller_(caller) {}
+    OnOwnStream(const OnOwnStream &) = delete;
+    ~OnOwnStream() { leave(); }
+    cudaError_t enter()
+    {
+        if (caller_ == c_->stream) return cudaSuccess;
+        cudaError_t e = cudaEventRecord(c_->ev_in, caller_);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(c_->stream, c_->ev_in, 0);
+        open_ = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t leave()
+    {
+        if (!open_) return cudaSuccess;
+        open_ = false;
+        const cudaError_t e = cudaEventRecord(c_->ev_out, c_->stream);
+        return e == cudaSuccess ? cudaStreamWaitEvent(caller_, c_->ev_out, 0) : e;
+    }
+
+private:
+    stereo_ctx *c_;
+    cudaStream_t caller_;
+    bool open_ = false;
+};
+
 // Batches up to this size launch their kernels directly: capturing them as a
 // graph and updating the last one in place takes host time that a batch in a row
 // of batches hides and a lone small one does not (two VGA pairs: 85 us alone
@@ -829,10 +861,8 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(us, &cap)) != cudaSuccess) return cuda_fail(c, e, "stream capture");
     if (cap != cudaStreamCaptureStatusNone) return cuda_fail(c, cudaErrorStreamCaptureUnsupported, "stream capture");
-    if (us != s) {
-        if ((e = cudaEventRecord(c->ev_in, us)) != cudaSuccess || (e = cudaStreamWaitEvent(s, c->ev_in, 0)) != cudaSuccess)
-            return cuda_fail(c, e, "stream ordering");
-    }
+    OnOwnStream own(c, us);
+    if ((e = own.enter()) != cudaSuccess) return cuda_fail(c, e, "stream ordering");
 
     // tile shape: fixed, remembered for this batch signature, or tuned now
     int tile = c->tile;
@@ -920,10 +950,7 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
         cudaGraphDestroy(graph);
         if ((e = cudaGraphLaunch(exec, s)) != cudaSuccess) return cuda_fail(c, e, "graph launch");
     }
-    if (us != s) {
-        if ((e = cudaEventRecord(c->ev_out, s)) != cudaSuccess || (e = cudaStreamWaitEvent(us, c->ev_out, 0)) != cudaSuccess)
-            return cuda_fail(c, e, "stream ordering");
-    }
+    if ((e = own.leave()) != cudaSuccess) return cuda_fail(c, e, "stream ordering");
     c->launches = launches;
     c->last_batch_tile = tile;
     return STEREO_OK;
@@ -1036,22 +1063,14 @@ int diff_common(stereo_ctx *c, int B, int W, int H, int D, const float *l, const
 // stream into the capture.
 cudaError_t diff_launch(stereo_ctx *c, const DiffArgs &a, cudaStream_t us)
 {
-    cudaStream_t s = c->stream;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(us, &st);
     if (e != cudaSuccess) return e;
     if (st != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
     if ((e = diff_setup()) != cudaSuccess) return e;
-    if (us != s) {
-        if ((e = cudaEventRecord(c->ev_in, us)) != cudaSuccess || (e = cudaStreamWaitEvent(s, c->ev_in, 0)) != cudaSuccess)
-            return e;
-    }
-    if ((e = diff_run(a, s)) != cudaSuccess) return e;
-    if (us != s) {
-        if ((e = cudaEventRecord(c->ev_out, s)) != cudaSuccess || (e = cudaStreamWaitEvent(us, c->ev_out, 0)) != cudaSuccess)
-            return e;
-    }
-    return cudaSuccess;
+    OnOwnStream own(c, us);
+    if ((e = own.enter()) != cudaSuccess || (e = diff_run(a, c->stream)) != cudaSuccess) return e;
+    return own.leave();
 }
 
 }  // namespace

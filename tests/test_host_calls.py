@@ -1,0 +1,78 @@
+"""What the entry points do on the host, on the CPU with a runtime that only
+writes down its calls."""
+import os
+import sys
+
+import pytest
+
+sys.path.insert(0, os.path.dirname(os.path.abspath(__file__)))
+import fake_api  # noqa: E402
+from paper_2212_00488_gb300 import _lib  # noqa: E402
+
+pytestmark = pytest.mark.skipif(not fake_api.available(), reason="needs the CUDA headers and g++")
+
+CALLER = 0x77       # the caller's stream
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    return fake_api.build(tmp_path_factory.mktemp("fake"))
+
+
+@pytest.fixture
+def fake(fake_lib, monkeypatch):
+    monkeypatch.setattr(_lib, "_lib", fake_lib)      # the binding's functions call the fake
+    fake_lib.fake_reset()
+    return fake_lib
+
+
+def _lines(fake):
+    return [ln.split() for ln in fake.fake_log().decode().splitlines()]
+
+
+def _context(**params):
+    p = _lib.stereo_default_params()
+    for k, v in params.items():
+        setattr(p, k, v)
+    return _lib.stereo_create(0, p)
+
+
+def _jobs(widths):
+    return [_lib.stereo_job(1, 1, w, 60, 16, 1, None, None, None) for w in widths]
+
+
+def _caller_waits_for_all(lines):
+    """The last launch is followed by an event of its stream that the caller's stream waits for."""
+    last = max(i for i, ln in enumerate(lines) if ln[0] in ("launch", "graph"))
+    own = lines[last][-1]
+    after = lines[last + 1:]
+    return any(a[0] == "record" and a[2] == own and ["wait", f"{CALLER:x}", a[1]] in after[i + 1:]
+               for i, a in enumerate(after))
+
+
+@pytest.mark.parametrize("fail", [None, 0, 1, 2, 3])
+@pytest.mark.parametrize("what", ["batch", "forward", "backward"])
+def test_caller_waits_for_what_was_queued_also_after_an_error(fake, what, fail):
+    # the kernels run on the context's stream; those queued before one fails still
+    # read the caller's inputs, so the caller's stream has to come after them
+    ctx = _context()
+    _lib.stereo_set_tile(ctx, 1)
+    fake.fake_reset()
+    if fail is not None:
+        fake.fake_fail_at(fail)
+
+    def call():
+        if what == "batch":
+            _lib.stereo_compute_batch(ctx, _jobs([80, 80]), CALLER)
+        elif what == "forward":
+            _lib.stereo_diff_forward(ctx, 1, 8, 8, 4, 1, 1, 1, 1, 1, 0.1, 1, 1, CALLER)
+        else:
+            _lib.stereo_diff_backward(ctx, 1, 8, 8, 4, 1, 1, 1, 1, 1, 0.1, 1, 1, 1, 1, 1, 1, CALLER)
+    if fail is None:
+        call()
+    else:
+        with pytest.raises(_lib.StereoError) as e:
+            call()
+        assert e.value.code == _lib.STEREO_ECUDA and "a call failed" in str(e.value)
+    assert _caller_waits_for_all(_lines(fake))
+    _lib.stereo_destroy(ctx)
