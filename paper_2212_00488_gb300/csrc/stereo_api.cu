@@ -780,6 +780,15 @@ std::string batch_signature(const stereo_ctx *c, const std::vector<FrameWs> &fw)
     snprintf(buf, sizeof buf, "%.200s sms%d wx%d wy%d scale%d ds%d |", name, c->num_sms, c->p.wx, c->p.wy,
              c->p.cost_scale, c->p.downscale);
     std::string sig = buf;
+    // the lambdas set the largest cost, which decides what fits and whether tiles
+    // 3 and 8 are their split forms (not written at the defaults, so that files
+    // saved without them stay good)
+    stereo_params d;
+    stereo_default_params(&d);
+    if (c->p.lambda_ad != d.lambda_ad || c->p.lambda_mc != d.lambda_mc) {
+        snprintf(buf, sizeof buf, " lambda %.17g %.17g |", c->p.lambda_ad, c->p.lambda_mc);
+        sig += buf;
+    }
     std::vector<std::string> parts;
     for (const FrameWs &f : fw) {
         snprintf(buf, sizeof buf, " %dx%dx%d", f.X, f.Y, f.D);
@@ -867,13 +876,18 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
     // tile shape: fixed, remembered for this batch signature, or tuned now
     int tile = c->tile;
     int launches = 0;
+    auto misfit = [&](int t) {          // the first job tile t does not fit, or n
+        int k = 0;
+        while (k < n && costagg_fits(b.job[k], t)) ++k;
+        return k;
+    };
     if (tile >= 0) {
-        for (int k = 0; k < n; ++k)
-            if (!costagg_fits(b.job[k], tile)) return fail(c, STEREO_EINVAL, "tile %d does not fit job %d", tile, k);
+        const int k = misfit(tile);
+        if (k < n) return fail(c, STEREO_EINVAL, "tile %d does not fit job %d", tile, k);
     } else {
         const std::string sig = batch_signature(c, fw);
         auto it = c->tune.find(sig);
-        if (it != c->tune.end()) {
+        if (it != c->tune.end() && misfit(it->second) == n) {   // (a loaded file may name any tile)
             tile = it->second;
         } else {
             // the autotuner: run the preparation once, then time each tile
@@ -882,9 +896,7 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
             float best = 0.f;
             for (int t = 0; t < kNumTiles; ++t) {
                 c->last_batch_tune_ms[t] = -1.f;
-                bool ok = true;
-                for (int k = 0; k < n && ok; ++k) ok = costagg_fits(b.job[k], t);
-                if (!ok) continue;
+                if (misfit(t) < n) continue;
                 float tmin = 0.f;
                 for (int rep = 0; rep < 3; ++rep) {
                     BatchArgs bt = b;

@@ -76,3 +76,46 @@ def test_caller_waits_for_what_was_queued_also_after_an_error(fake, what, fail):
         assert e.value.code == _lib.STEREO_ECUDA and "a call failed" in str(e.value)
     assert _caller_waits_for_all(_lines(fake))
     _lib.stereo_destroy(ctx)
+
+
+def _tile_of(ctx, jobs):
+    _lib.stereo_compute_batch(ctx, jobs, CALLER)
+    return _lib.stereo_batch_tile(ctx)[0]
+
+
+def test_a_remembered_tile_holds_for_its_matching_costs_only(fake, tmp_path):
+    # at wx 33 the 16-bit tile fits the default costs (67 P < 2^16) and not those
+    # of lambda_ad 0.2: the other context's choice must not be taken for its own
+    path = str(tmp_path / "tune.txt")
+    a, b = _context(wx=33), _context(wx=33, lambda_ad=0.2)
+    jobs = _jobs([80])
+    assert _tile_of(a, jobs) == 0
+    assert _lib.stereo_tune_save(a, path) == 1
+    assert _lib.stereo_tune_load(b, path) == 1
+    assert _tile_of(b, jobs) == 1
+    # each finds its own choice again, without tuning, from one file
+    assert _lib.stereo_tune_save(b, path) == 2
+    for params, tile in ((dict(wx=33), 0), (dict(wx=33, lambda_ad=0.2), 1)):
+        c = _context(**params)
+        assert _lib.stereo_tune_load(c, path) == 2
+        fake.fake_reset()
+        assert _tile_of(c, jobs) == tile
+        assert sum(ln[:2] == ["launch", "batch"] for ln in _lines(fake)) == 1
+        _lib.stereo_destroy(c)
+    _lib.stereo_destroy(a)
+    _lib.stereo_destroy(b)
+
+
+def test_a_remembered_tile_that_does_not_fit_is_tuned_again(fake, tmp_path):
+    path = tmp_path / "tune.txt"
+    a = _context(wx=40)                     # 81 P > 2^16: not the 16-bit tile
+    jobs = _jobs([80])
+    assert _tile_of(a, jobs) == 1
+    _lib.stereo_tune_save(a, str(path))
+    sig = path.read_text().split("\t")[0]
+    path.write_text(f"{sig}\t0\n")
+    c = _context(wx=40)
+    assert _lib.stereo_tune_load(c, str(path)) == 1
+    assert _tile_of(c, jobs) == 1
+    _lib.stereo_destroy(a)
+    _lib.stereo_destroy(c)
