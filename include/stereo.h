@@ -228,7 +228,9 @@ typedef struct {
 
 /* Up to 32 pairs in one call (the batched form of the method; the paper
  * processes one pair at a time). Preparation and post-processing take one
- * launch a step for all frames, the fused cost + aggregation + WTA of all
+ * launch a step for all frames (the grey conversion two where the rows of some
+ * frames are word-aligned and those of others are not, and one a frame without
+ * downscaling), the fused cost + aggregation + WTA of all
  * frames runs as one persistent kernel taking (frame, strip, slab) tiles
  * largest frame first; a batch of more than four frames is one CUDA graph,
  * re-captured and updated in place on each call, a smaller one is launched

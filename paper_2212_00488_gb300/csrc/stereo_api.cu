@@ -11,6 +11,7 @@
 #include <map>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 using namespace stereo;
@@ -78,7 +79,8 @@ struct stereo_ctx {
     // the autotuner's choices of tile shape per batch signature.
     void *bws = nullptr;
     size_t bws_size = 0;
-    std::map<int, cudaGraphExec_t> bexec;   // one graph per batch size, updated in place
+    // one graph per batch size and number of launches (its topology), updated in place
+    std::map<std::pair<int, int>, cudaGraphExec_t> bexec;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr, ev_t0 = nullptr, ev_t1 = nullptr;
     std::map<std::string, int> tune;
     void *dws = nullptr;            // workspace of the differentiable form
@@ -943,9 +945,10 @@ int stereo_compute_batch(stereo_ctx *c, int n, const stereo_job *jobs, void *str
             cudaGetLastError();
             return cuda_fail(c, e != cudaSuccess ? e : e2, "batch capture");
         }
-        // batches of one size share the graph topology, so the last graph of that
-        // size is updated in place; a new size or tile shape instantiates anew
-        cudaGraphExec_t &exec = c->bexec[n];
+        // batches of one size and number of launches (one grey launch, or two where
+        // some frames' rows are word-aligned and others' not) share the graph topology:
+        // their last graph is updated in place
+        cudaGraphExec_t &exec = c->bexec[{n, launches}];
         if (exec) {
             cudaGraphExecUpdateResultInfo info;
             if (cudaGraphExecUpdate(exec, graph, &info) != cudaSuccess) {

@@ -119,3 +119,19 @@ def test_a_remembered_tile_that_does_not_fit_is_tuned_again(fake, tmp_path):
     assert _tile_of(c, jobs) == 1
     _lib.stereo_destroy(a)
     _lib.stereo_destroy(c)
+
+
+def test_batches_of_aligned_and_of_mixed_frames_keep_a_graph_each(fake):
+    # frames whose rows are word-aligned and others take a grey launch each, so
+    # batches of one size come in two topologies; taking them in turn must not
+    # instantiate a graph again on every call
+    ctx = _context()
+    _lib.stereo_set_tile(ctx, 1)
+    fake.fake_reset()
+    for _ in range(3):
+        for widths in ([80] * 6, [80] * 3 + [81] * 3, [81] * 6):
+            _lib.stereo_compute_batch(ctx, _jobs(widths), CALLER)
+    lines = _lines(fake)
+    assert sum(ln[0] == "graph" for ln in lines) == 9
+    assert sum(ln[0] == "instantiate" for ln in lines) == 2
+    _lib.stereo_destroy(ctx)
