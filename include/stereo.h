@@ -313,8 +313,8 @@ STEREO_API int stereo_diff_backward(stereo_ctx *ctx, int B, int W, int H, int D,
  * All intermediates live in one fixed 32 MiB device array inside the library,
  * which every GPU that loads the library holds until the process exits. A
  * frame fits when its workspace does: with the default parameters that is
- * about 11.8 bytes per input pixel with downscaling (1436x992 needs 17 MB; up
- * to about 2.8 Mpixel) and about 43 bytes per pixel without it (up to about
+ * about 10.9 bytes per input pixel with downscaling (1436x992 needs 15.5 MB; up
+ * to about 3 Mpixel) and about 43 bytes per pixel without it (up to about
  * 0.78 Mpixel). A larger frame is rejected with STEREO_ENOMEM and a message in
  * err. Nothing is allocated: no cudaMalloc, cudaFree or allocating library
  * call.

@@ -43,7 +43,6 @@ constexpr int kMaxWx = 141;    // the largest W_x of Table I
 
 struct CostAggArgs {
     const uint32_t *pix_l, *pix_r;   // [Y][X]
-    const uint32_t *arm_l, *arm_r;   // [Y][X]
     const uint32_t *armc_l, *armc_r; // armc_words(X, Y, wy), laid out by armc_index
     uint32_t *key_l, *key_r;         // [Y][X] min over d of (CA << 8 | d); preset to ~0
     const uint32_t *lut_ad;          // [256] quantised AD cost (Eq. 4) by |grey difference|

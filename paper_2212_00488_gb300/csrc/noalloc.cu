@@ -86,7 +86,7 @@ extern "C" int stereo_compute_noalloc(const stereo_params *params, const uint8_t
     auto take = [&](size_t bytes) { size_t o = off; off += up256(bytes); return o; };
     const size_t o_lut = take(264 * 4), o_err = take(4);
     size_t o_gf[2], o_gs[2], o_pix[2], o_arm[2], o_armc[2], o_key[2];
-    for (int i = 0; i < 2; ++i) o_gf[i] = take(nf);
+    for (int i = 0; i < 2; ++i) o_gf[i] = ds && i ? 0 : take(nf);   // (downscaling keeps the left image's only)
     for (int i = 0; i < 2; ++i) o_gs[i] = ds ? take(nl) : o_gf[i];
     for (int i = 0; i < 2; ++i) o_pix[i] = take(nl * 4);
     for (int i = 0; i < 2; ++i) o_arm[i] = take(nl * 4);
@@ -133,8 +133,6 @@ extern "C" int stereo_compute_noalloc(const stereo_params *params, const uint8_t
         CostAggArgs a{};
         a.pix_l = u32(o_pix[0]);
         a.pix_r = u32(o_pix[1]);
-        a.arm_l = u32(o_arm[0]);
-        a.arm_r = u32(o_arm[1]);
         a.armc_l = u32(o_armc[0]);
         a.armc_r = u32(o_armc[1]);
         a.key_l = u32(o_key[0]);

@@ -36,7 +36,7 @@ struct stereo_ctx {
     // layout of the current frame inside ws
     int W = 0, H = 0, Dmax = 0, X = 0, Y = 0, D = 0;
     bool host_staging = false;
-    uint8_t *gf[2] = {nullptr, nullptr};   // full-res grey (the processed grey without downscaling)
+    uint8_t *gf[2] = {nullptr, nullptr};   // full-res grey (left only with downscaling, the processed grey without)
     uint8_t *gs[2] = {nullptr, nullptr};   // processed grey
     uint32_t *pix[2] = {nullptr, nullptr};
     uint32_t *arm[2] = {nullptr, nullptr};
@@ -175,7 +175,7 @@ size_t layout(stereo_ctx *c, char *base, int W, int H, bool staging)
         off += align256(bytes);
         return p;
     };
-    for (int i = 0; i < 2; ++i) c->gf[i] = (uint8_t *)take(nf);
+    for (int i = 0; i < 2; ++i) c->gf[i] = ds && i ? nullptr : (uint8_t *)take(nf);
     for (int i = 0; i < 2; ++i) c->gs[i] = ds ? (uint8_t *)take(nl) : c->gf[i];
     for (int i = 0; i < 2; ++i) c->pix[i] = (uint32_t *)take(nl * 4);
     for (int i = 0; i < 2; ++i) c->arm[i] = (uint32_t *)take(nl * 4);
@@ -264,8 +264,6 @@ cudaError_t run_stage(stereo_ctx *c, int stage, cudaStream_t s)
         CostAggArgs a;
         a.pix_l = c->pix[0];
         a.pix_r = c->pix[1];
-        a.arm_l = c->arm[0];
-        a.arm_r = c->arm[1];
         a.armc_l = c->armc[0];
         a.armc_r = c->armc[1];
         a.key_l = c->key[0];
@@ -654,7 +652,7 @@ size_t frame_layout(const stereo_params &p, int W, int H, int Dmax, char *base, 
     g.X = X;
     g.Y = Y;
     g.D = ds ? (Dmax + 1) / 2 : Dmax;
-    for (int i = 0; i < 2; ++i) g.gf[i] = (uint8_t *)take(nf);
+    for (int i = 0; i < 2; ++i) g.gf[i] = ds && i ? nullptr : (uint8_t *)take(nf);
     for (int i = 0; i < 2; ++i) g.gs[i] = ds ? (uint8_t *)take(nl) : g.gf[i];
     for (int i = 0; i < 2; ++i) g.pix[i] = (uint32_t *)take(nl * 4);
     for (int i = 0; i < 2; ++i) g.arm[i] = (uint32_t *)take(nl * 4);
@@ -671,8 +669,6 @@ CostAggArgs frame_args(const stereo_ctx *c, const FrameWs &f)
     CostAggArgs a{};
     a.pix_l = f.pix[0];
     a.pix_r = f.pix[1];
-    a.arm_l = f.arm[0];
-    a.arm_r = f.arm[1];
     a.armc_l = f.armc[0];
     a.armc_r = f.armc[1];
     a.key_l = f.key[0];

@@ -135,3 +135,16 @@ def test_batches_of_aligned_and_of_mixed_frames_keep_a_graph_each(fake):
     assert sum(ln[0] == "graph" for ln in lines) == 9
     assert sum(ln[0] == "instantiate" for ln in lines) == 2
     _lib.stereo_destroy(ctx)
+
+
+@pytest.mark.parametrize("downscale", [0, 1])
+def test_a_frame_takes_the_planes_it_uses(fake, downscale):
+    p = _lib.stereo_default_params()
+    p.downscale = downscale
+    W, H = 642, 481
+    X, Y = (W // 2, H // 2) if downscale else (W, H)
+    n = X * Y
+    # full-res grey of the left image beside both processed ones, or the processed ones alone; pixel and arm
+    # words, the fused kernel's arm words (whole row quads), keys; medians and filled map
+    planes = [W * H] * downscale + [n] * 2 + [4 * n] * 6 + [4 * X * ((Y + p.wy + 3) // 4 * 4)] * 2 + [n, 4 * n]
+    assert _lib.stereo_job_bytes(p, W, H, 64) == sum((b + 255) // 256 * 256 for b in planes) + 256
