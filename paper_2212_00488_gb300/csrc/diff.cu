@@ -769,12 +769,12 @@ __global__ void __launch_bounds__(kRedNT) diff_theta_reduce_kernel(const double 
 struct DiffWs {
     float *gl, *gr;
     uint8_t *ql, *qr;
-    uint32_t *pixl, *pixr, *arml, *armr, *armcl, *armcr, *keyl, *keyr;
-    float *ns, *state, *accl, *accr, *s0, *s1, *s2, *s3, *part;
+    uint32_t *pixl, *pixr, *arml;
+    float *ns, *state, *accl, *accr, *s0, *s1, *s2, *part;
     double *seg;
 };
 
-size_t diff_layout(char *base, int X, int Y, int wy, int B, int D, DiffWs *w)
+size_t diff_layout(char *base, int X, int Y, int B, int D, DiffWs *w)
 {
     const size_t n = (size_t)X * Y, nb = (size_t)B;
     const size_t nchunks = (D + kDC - 1) / kDC;
@@ -789,31 +789,25 @@ size_t diff_layout(char *base, int X, int Y, int wy, int B, int D, DiffWs *w)
     t.gr = (float *)take(nb * n * 4);
     t.ql = (uint8_t *)take(nb * n);                          // integer grey of the uint8 images
     t.qr = (uint8_t *)take(nb * n);
-    t.pixl = (uint32_t *)take(nb * n * 4);                   // pixel and arm words
+    t.pixl = (uint32_t *)take(nb * n * 4);                   // pixel words, arm words of the left images
     t.pixr = (uint32_t *)take(nb * n * 4);
     t.arml = (uint32_t *)take(nb * n * 4);
-    t.armr = (uint32_t *)take(nb * n * 4);
-    t.armcl = (uint32_t *)take(nb * armc_words(X, Y, wy) * 4);
-    t.armcr = (uint32_t *)take(nb * armc_words(X, Y, wy) * 4);
-    t.keyl = (uint32_t *)take(nb * n * 4);                   // keys (written by the support pass)
-    t.keyr = (uint32_t *)take(nb * n * 4);
     t.ns = (float *)take(nb * n * 4);                        // support size
     t.state = (float *)take(nb * n * 4 * 3);                 // online softmax state
     t.accl = (float *)take(nb * n * 4);                      // intensity-gradient accumulators
     t.accr = (float *)take(nb * n * 4);
-    t.s0 = (float *)take(nb * kDC * n * 4);                  // slabs
+    t.s0 = (float *)take(nb * kDC * n * 4);                  // slabs: x sums, their gradient, its vertical adjoint
     t.s1 = (float *)take(nb * kDC * n * 4);
     t.s2 = (float *)take(nb * kDC * n * 4);
-    t.s3 = (float *)take(nb * kDC * n * 4);
     t.part = (float *)take(nb * nchunks * hgrad_blocks(X, Y) * 16);   // parameter-gradient partials
     t.seg = (double *)take(kRedBlocks * 4 * sizeof(double)); // their segment sums
     if (w) *w = t;
     return off;
 }
 
-size_t diff_workspace_bytes(int X, int Y, int wy, int B, int D)
+size_t diff_workspace_bytes(int X, int Y, int B, int D)
 {
-    return diff_layout(nullptr, X, Y, wy, B, D, nullptr);
+    return diff_layout(nullptr, X, Y, B, D, nullptr);
 }
 
 cudaError_t diff_setup()
@@ -830,7 +824,7 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
 {
     const int X = a.W, Y = a.H, n = X * Y, B = a.B;
     DiffWs w;
-    diff_layout((char *)a.ws, X, Y, a.wy, B, a.D, &w);
+    diff_layout((char *)a.ws, X, Y, B, a.D, &w);
     const int nblk = (n + kDiffNT - 1) / kDiffNT;
     const int nchunks = (a.D + kDC - 1) / kDC;
     const int nseg = hgrad_segments(X), yblocks = (Y + kHRows - 1) / kHRows;

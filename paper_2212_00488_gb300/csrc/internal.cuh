@@ -113,11 +113,11 @@ struct DiffArgs {
     float *grad_left, *grad_right;     // backward only, [B][H][W][3]
     float *grad_theta;                 // backward only, [4]
     int backward;
-    void *ws;                          // diff_workspace_bytes(W, H, wy, B, D) bytes
+    void *ws;                          // diff_workspace_bytes(W, H, B, D) bytes
     uint32_t *err;
     int wx, wy, tc;
 };
-size_t diff_workspace_bytes(int X, int Y, int wy, int B, int D);
+size_t diff_workspace_bytes(int X, int Y, int B, int D);
 // Sets the differentiable kernels' attributes on the current device (call
 // before diff_run and outside any stream capture).
 cudaError_t diff_setup();

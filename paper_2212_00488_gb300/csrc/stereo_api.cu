@@ -1030,7 +1030,7 @@ int diff_common(stereo_ctx *c, int B, int W, int H, int D, const float *l, const
     if (!l || !r || !lu || !ru || !theta) return fail(c, STEREO_EINVAL, "NULL input");
     if (B < 1 || B > 64 || W < 1 || H < 1 || W > 4096 || H > 8192 || D < 1 || D > 256 || !(tau > 0.f))
         return fail(c, STEREO_EINVAL, "bad B, W, H, D or tau");
-    const size_t need = diff_workspace_bytes(W, H, c->p.wy, B, D);
+    const size_t need = diff_workspace_bytes(W, H, B, D);
     if (need > c->dws_size) {
         if (c->mem_cap && need + c->ws_size + c->bws_size > c->mem_cap)
             return fail(c, STEREO_ENOMEM, "differentiable workspace of %zu bytes exceeds the cap", need);

@@ -82,7 +82,7 @@ cudaError_t launch_unpack_planes(const uint32_t *, const uint32_t *, uint8_t *, 
 {
     return launch("unpack", s);
 }
-size_t diff_workspace_bytes(int, int, int, int, int) { return 256; }
+size_t diff_workspace_bytes(int, int, int, int) { return 256; }
 cudaError_t diff_run(const DiffArgs &, cudaStream_t s)
 {
     for (int i = 0; i < 4; ++i) {

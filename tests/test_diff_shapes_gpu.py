@@ -87,3 +87,30 @@ def _check(B, W, H, D, wx, wy, seed=0):
                                         (3, 4, 4, 256, 0), (8, 3, 8, 256, 0)])
 def test_images_of_a_few_pixels(B, W, H, D, wy):
     _check(B, W, H, D, 21, wy)
+
+
+def test_workspace_holds_only_planes_in_use():
+    # 142 bytes a pixel and pair, and the partials (16 bytes for two rows of a
+    # segment and chunk): a context capped at 150 bytes a pixel runs the step
+    from paper_2212_00488_gb300 import Stereo, _lib
+    from paper_2212_00488_gb300.diff import soft_argmin_disparity
+    B, W, H, D = 2, 300, 200, 24
+    lu, ru, go = _grey_images(B, W, H, 3)
+    res = []
+    for cap in (0, 150 * B * W * H):
+        st = Stereo(0, downscale=0, mem_cap_bytes=cap)
+        l, r = (torch.from_numpy(a.astype(np.float32) / 255).cuda().requires_grad_(True) for a in (lu, ru))
+        theta = torch.tensor(THETA, device="cuda", requires_grad=True)
+        dhat = soft_argmin_disparity(l, r, theta, torch.from_numpy(lu).cuda(), torch.from_numpy(ru).cuda(), D, TAU, st)
+        res.append((dhat.detach(), *torch.autograd.grad(dhat.sum(), (l, r, theta))))
+        torch.cuda.synchronize()
+        st.close()
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+    st = Stereo(0, downscale=0, mem_cap_bytes=100 * B * W * H)
+    with pytest.raises(_lib.StereoError) as e:
+        soft_argmin_disparity(*(torch.from_numpy(a.astype(np.float32)).cuda() for a in (lu, ru)),
+                              torch.tensor(THETA, device="cuda"), torch.from_numpy(lu).cuda(),
+                              torch.from_numpy(ru).cuda(), D, TAU, st)
+    assert e.value.code == _lib.STEREO_ENOMEM
+    st.close()
