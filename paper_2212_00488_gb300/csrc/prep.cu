@@ -197,7 +197,8 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__
 // byte compare, so a step costs six instructions for four pixels whatever the
 // arms' lengths. The four rows of a quad go through a step together, which
 // hides the latency of each, and a warp stops when none of its 512 arms goes
-// on (tested every four steps). Bound by the ALU pipe. At 718 x 496 (two
+// on (tested every four steps) or can: the staged pixels beyond the image repeat its
+// border, so an arm that reaches it would never end there by itself. Bound by the ALU pipe. At 718 x 496 (two
 // images) 34.5 us with one thread following each arm eight pixels at a time
 // and a queue for the arms that go on, 16.5 us now (cold L2, both).
 constexpr int kSX = 128, kSY = 16;           // pixels of a CTA
@@ -291,9 +292,10 @@ __device__ __forceinline__ void arm_step(uint32_t w, uint32_t c, uint32_t bm, ui
 }
 
 // Horizontal arms of a lane's four pixels in four rows: `row` is the lane's
-// word of the first row, `pitch` the row pitch; kDir -1 left, +1 right.
+// word of the first row, `pitch` the row pitch; kDir -1 left, +1 right. No pixel of
+// the lane has more than `room` pixels of the image in that direction.
 template <bool kBig, int kDir>
-__device__ __forceinline__ void scan_x(const uint32_t *row, int pitch, int cap, uint32_t bm, uint32_t (&n)[4])
+__device__ __forceinline__ void scan_x(const uint32_t *row, int pitch, int cap, int room, uint32_t bm, uint32_t (&n)[4])
 {
     uint32_t c[4], cur[4], dead[4];
 #pragma unroll
@@ -315,7 +317,7 @@ __device__ __forceinline__ void scan_x(const uint32_t *row, int pitch, int cap, 
             }
             cur[j] = nx;
         }
-        if (__all_sync(0xffffffffu, (dead[0] & dead[1] & dead[2] & dead[3] & kHi) == kHi)) break;
+        if (__all_sync(0xffffffffu, (dead[0] & dead[1] & dead[2] & dead[3] & kHi) == kHi || t + 4 >= room)) break;
     }
 }
 
@@ -388,13 +390,13 @@ __global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_co
         uint32_t n[4];
         const uint32_t *rw = rows + (1 + 4 * q) * RW + hw + lane, *cl = cols + (wy + 4 * q) * P + lane;
         if (dir == 0)
-            scan_x<kBig, -1>(rw, RW, wx, bm, n);
+            scan_x<kBig, -1>(rw, RW, wx, x0 + 4 * lane < X ? x0 + 4 * lane + 3 : 0, bm, n);
         else if (dir == 1)
-            scan_x<kBig, 1>(rw, RW, wx, bm, n);
+            scan_x<kBig, 1>(rw, RW, wx, X - 1 - (x0 + 4 * lane), bm, n);
         else if (dir == 2)
-            scan_y<kBig, -1>(cl, wy, bm, n);
+            scan_y<kBig, -1>(cl, min(wy, y0 + 4 * q + 3), bm, n);
         else
-            scan_y<kBig, 1>(cl, wy, bm, n);
+            scan_y<kBig, 1>(cl, min(wy, Y - 1 - (y0 + 4 * q)), bm, n);
 #pragma unroll
         for (int j = 0; j < 4; ++j) res[(dir * kSY + 4 * q + j) * P + lane] = n[j];
     }
