@@ -620,23 +620,16 @@ __host__ __device__ __forceinline__ int slab_strips(const CostAggArgs &a, int sl
     return (a.X + d0 - right_shift<T>(a, d0) + T::XS - 1) / T::XS;
 }
 
-template <class T>
-__host__ __device__ __forceinline__ int tiles_of(const CostAggArgs &a)
-{
-    int n = 0;
-    for (int s = 0; s * T::DS < a.D; ++s) n += slab_strips<T>(a, s);
-    return n;
-}
-
-// CTA t of a frame: the first a.head tiles (strip, slab) are swept from the first
-// row to the last, the others in row bands of a.band rows: all of them in the
-// first band, then in the next.
+// CTA t of a frame: the first a.head tiles (strip, slab) of a.tiles are swept from
+// the first row to the last, the others in row bands of a.band rows: all of them
+// in the first band, then in the next. (The count comes with the arguments: adding
+// it up over the slabs cost a CTA 1.2 us at 26 slabs.)
 template <class T>
 __device__ __forceinline__ void run_tile(const CostAggArgs &a, int t, unsigned char *smem, bool reuse)
 {
     int ya = 0, yb = a.Y;
     if (t >= a.head) {
-        const int rest = tiles_of<T>(a) - a.head, band = (t - a.head) / rest;
+        const int rest = a.tiles - a.head, band = (t - a.head) / rest;
         t -= band * rest;
         ya = band * a.band;
         yb = min(ya + a.band, a.Y);
@@ -758,6 +751,14 @@ cudaError_t setup_one()
     return cudaFuncSetAttribute(costagg_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::BYTES);
 }
 
+template <class T>
+int tiles_of(const CostAggArgs &a)
+{
+    int n = 0;
+    for (int s = 0; s * T::DS < a.D; ++s) n += slab_strips<T>(a, s);
+    return n;
+}
+
 // Row steps of one tile when a frame of Y rows is cut into bands of `band` rows
 // (a multiple of 4): the band, the wy rows its windows reach above and below
 // it, and about 40 rows' worth of start-up (table, first rows, launch).
@@ -773,8 +774,10 @@ constexpr int kMaxBands = 8;
 template <class T>
 cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
 {
-    for (int j = 0; j < b.njobs; ++j)
+    for (int j = 0; j < b.njobs; ++j) {
         if (!fits<T>(b.job[j])) return cudaErrorInvalidValue;
+        b.job[j].tiles = tiles_of<T>(b.job[j]);
+    }
     // bands where the frames' tiles leave SMs idle: few tiles go in rounds over
     // the SMs, many even out and leave about half a long tile at the end
     double best = 0;
@@ -785,7 +788,7 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
         for (int j = 0; j < b.njobs; ++j) {
             const CostAggArgs &a = b.job[j];
             const int rows = band_rows(a, n), steps = band_steps(a, rows);
-            const long nt = (long)tiles_of<T>(a) * ((a.Y + rows - 1) / rows);
+            const long nt = (long)a.tiles * ((a.Y + rows - 1) / rows);
             tiles += nt;
             sum += (double)nt * steps;
             last = std::max(last, (double)steps);
@@ -803,7 +806,7 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
         a.band = band_rows(a, nb);
         a.head = 0;
         b.tile_start[j] = b.total_tiles;
-        b.total_tiles += tiles_of<T>(a) * ((a.Y + a.band - 1) / a.band);
+        b.total_tiles += a.tiles * ((a.Y + a.band - 1) / a.band);
     }
     b.tile_start[b.njobs] = b.total_tiles;
     cudaError_t e = cudaMemsetAsync(b.counter, 0, sizeof(uint32_t), s);
@@ -847,7 +850,8 @@ template <class T>
 cudaError_t launch_one(CostAggArgs a, cudaStream_t s)
 {
     estimate<T>(a, a.num_sms, a.head, a.band);
-    const int ctas = a.head + (tiles_of<T>(a) - a.head) * ((a.Y + a.band - 1) / a.band);
+    a.tiles = tiles_of<T>(a);
+    const int ctas = a.head + (a.tiles - a.head) * ((a.Y + a.band - 1) / a.band);
     return launch_dependent(costagg_wta_kernel<T>, dim3(ctas), dim3(T::NT), T::BYTES, s, a);
 }
 

@@ -54,7 +54,8 @@ struct CostAggArgs {
     uint32_t P;                      // cost of a match outside the image
     int tile;                        // tile shape id, -1 = pick from the shape
     int num_sms;                     // SMs of the device (for the pick)
-    int head, band;                  // tiles swept in one piece, rows of the others' bands (filled by the launcher)
+    int tiles, head, band;           // tiles of the frame, those swept in one piece, rows of the others' bands (filled by
+                                     // the launcher)
 };
 
 // Programmatic dependent launch between the kernels of a frame: a kernel
