@@ -751,11 +751,21 @@ cudaError_t setup_one()
     return cudaFuncSetAttribute(costagg_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::BYTES);
 }
 
+// Tiles of a frame: the strips of all slabs (slab_strips). Neighbouring slabs
+// mostly have the same number of strips, so they are counted in runs of equal ones.
 template <class T>
 int tiles_of(const CostAggArgs &a)
 {
-    int n = 0;
-    for (int s = 0; s * T::DS < a.D; ++s) n += slab_strips<T>(a, s);
+    const int last = (a.D - 1) / T::DS;                       // the last slab, on its own: it may overlap
+    int n = slab_strips<T>(a, last);
+    for (int s = 0; s < last;) {
+        const int strips = slab_strips<T>(a, s);
+        // the columns to cover grow by the disparities past right_shift's spare entries
+        const int spare = T::NE - (T::XS + T::DS - 1 + 2 * a.wx);
+        const int end = std::min(last, (strips * T::XS - a.X + spare) / T::DS + 1);   // first slab with more
+        n += strips * (end - s);
+        s = end;
+    }
     return n;
 }
 
@@ -770,6 +780,24 @@ int band_steps(const CostAggArgs &a, int band)
 int band_rows(const CostAggArgs &a, int nb) { return ((a.Y + nb - 1) / nb + 3) / 4 * 4; }
 
 constexpr int kMaxBands = 8;
+
+// The ways a frame's tiles can be cut into bands; they do not depend on the tile
+// shape, so the pick works them out once.
+struct Cuts {
+    int n = 0;
+    int rows[kMaxBands], bands[kMaxBands], steps[kMaxBands];
+    int whole;                                                // row steps of a tile in one piece
+    explicit Cuts(const CostAggArgs &a) : whole(band_steps(a, a.Y))
+    {
+        for (int nb = 1; nb <= kMaxBands; ++nb) {
+            const int r = band_rows(a, nb);
+            if (n && r == rows[n - 1]) continue;
+            rows[n] = r;
+            bands[n] = (a.Y + r - 1) / r;
+            steps[n++] = band_steps(a, r);
+        }
+    }
+};
 
 template <class T>
 cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
@@ -817,7 +845,7 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
 }
 
 // Time of a frame in ns with this tile in its best cut, waves of CTAs times their
-// row steps times the tile's measured time per step; sets the cut. A small
+// row steps times the tile's measured time per step; sets the tile count and the cut. A small
 // frame's tiles leave SMs idle: all of them go in bands (360 x 248 x 36: 38.1 us
 // in one band, 56 CTAs of 152 SMs, 17.8 us cut). A larger frame's last wave does:
 // whole waves of tiles stay in one piece, without the wy rows a band sweeps above
@@ -825,21 +853,20 @@ cudaError_t launch_batch_one(BatchArgs &b, int nsm, cudaStream_t s)
 // all in two bands 140 us, 152 whole and 19 in bands 106; 3840 x 2160, 4.4
 // waves: 707 and 644 us).
 template <class T>
-double estimate(const CostAggArgs &a, int nsm, int &head, int &band)
+int64_t estimate(CostAggArgs &a, const Cuts &cuts, int nsm)
 {
-    const int tiles = tiles_of<T>(a), waves = tiles / nsm;
-    double best = 0;
-    head = -1;
-    for (int k : {0, waves}) {
-        const int rest = tiles - k * nsm;
-        for (int n = 1; n <= kMaxBands; ++n) {
-            const int rows = band_rows(a, n);
-            const long ctas = (long)rest * ((a.Y + rows - 1) / rows);
-            const double t = ((double)k * band_steps(a, a.Y) + (double)((ctas + nsm - 1) / nsm) * band_steps(a, rows)) * T::NS;
-            if (head < 0 || t < best) {
+    a.tiles = tiles_of<T>(a);
+    const int waves = a.tiles / nsm;
+    int64_t best = -1;
+    for (int k = 0; k <= waves; k += std::max(waves, 1)) {    // none or all full waves whole
+        const int rest = a.tiles - k * nsm;
+        for (int i = 0; i < cuts.n; ++i) {
+            const int rounds = (rest * cuts.bands[i] + nsm - 1) / nsm;
+            const int64_t t = ((int64_t)k * cuts.whole + (int64_t)rounds * cuts.steps[i]) * T::NS;
+            if (best < 0 || t < best) {
                 best = t;
-                head = k * nsm;
-                band = rows;
+                a.head = k * nsm;
+                a.band = cuts.rows[i];
             }
         }
     }
@@ -847,10 +874,8 @@ double estimate(const CostAggArgs &a, int nsm, int &head, int &band)
 }
 
 template <class T>
-cudaError_t launch_one(CostAggArgs a, cudaStream_t s)
+cudaError_t launch_one(const CostAggArgs &a, cudaStream_t s)
 {
-    estimate<T>(a, a.num_sms, a.head, a.band);
-    a.tiles = tiles_of<T>(a);
     const int ctas = a.head + (a.tiles - a.head) * ((a.Y + a.band - 1) / a.band);
     return launch_dependent(costagg_wta_kernel<T>, dim3(ctas), dim3(T::NT), T::BYTES, s, a);
 }
@@ -866,22 +891,39 @@ cudaError_t costagg_setup()
     return e;
 }
 
-int costagg_pick(const CostAggArgs &a, int nsm)
+namespace {
+
+// The tile of a frame (a.tile, or the one with the least time), with its cut set; -1: none fits.
+int pick(CostAggArgs &a, int nsm)
 {
+    const Cuts cuts(a);
+    const bool split = split_fits(a);
     int best = -1;
-    double bt = 0;
-    for (int id = 0; id < kNumTiles; ++id)
-        with_tile(id, split_fits(a), [&](auto tag) {
+    int64_t bt = 0;
+    CostAggArgs c = a;
+    for (int id = std::max(a.tile, 0); id < (a.tile >= 0 ? a.tile + 1 : kNumTiles); ++id)
+        with_tile(id, split, [&](auto tag) {
             using T = typename decltype(tag)::type;
-            if (!fits<T>(a)) return;
-            int head, band;
-            const double est = estimate<T>(a, nsm, head, band);
-            if (best < 0 || est < bt) {
+            if (!fits<T>(c)) return;
+            const int64_t t = estimate<T>(c, cuts, nsm);
+            if (best < 0 || t < bt) {
                 best = id;
-                bt = est;
+                bt = t;
+                a.tiles = c.tiles;
+                a.head = c.head;
+                a.band = c.band;
             }
         });
     return best;
+}
+
+}  // namespace
+
+int costagg_pick(const CostAggArgs &a, int nsm)
+{
+    CostAggArgs c = a;
+    c.tile = -1;
+    return pick(c, nsm);
 }
 
 bool costagg_fits(const CostAggArgs &a, int tile)
@@ -903,12 +945,10 @@ cudaError_t launch_costagg_batch(BatchArgs &b, int tile, int nsm, cudaStream_t s
 cudaError_t launch_costagg(const CostAggArgs &a, cudaStream_t s)
 {
     if (a.wy > kMaxWy || a.wy < 0 || a.wx < 0 || a.wx > kMaxWx) return cudaErrorInvalidValue;
-    const int tile = a.tile >= 0 ? a.tile : costagg_pick(a, a.num_sms);
+    CostAggArgs c = a;
+    const int tile = pick(c, a.num_sms);
     cudaError_t e = cudaErrorInvalidValue;
-    with_tile(tile, split_fits(a), [&](auto tag) {
-        using T = typename decltype(tag)::type;
-        if (fits<T>(a)) e = launch_one<T>(a, s);
-    });
+    with_tile(tile, split_fits(a), [&](auto tag) { e = launch_one<typename decltype(tag)::type>(c, s); });
     return e;
 }
 
