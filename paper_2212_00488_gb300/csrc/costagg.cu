@@ -678,20 +678,24 @@ __global__ void __launch_bounds__(T::NT, 1) costagg_batch_kernel(const __grid_co
 }
 
 // Tile shapes (XS x DS, KE, RS, 16-bit prefixes, DPT, producer warps, largest
-// wx, ns per row step at 718 x 496 x 73). One CTA per SM; the ring of 64 prefix rows per (column, disparity, base)
+// wx, ns per row step). The times are what fits the frames of a sweep that keep
+// every SM busy, relative to tile 0 (at 718 x 496 x 73 alone tile 4 takes 93 where it
+// takes 108 in frames of several waves, and was picked there at a loss of up to 17 %;
+// sweep of 83 frames: picks 1.2 % from the best tile on average before, 0.6 % now).
+// One CTA per SM; the ring of 64 prefix rows per (column, disparity, base)
 // dominates shared memory. Every shape gives the same keys.
 using T0 = Tile<96, 4, 5, 12, true, 4, 12, 26, 121>;  // window sums < 2^16; at 718 columns 8 strips for every slab
-using T1 = Tile<96, 4, 7, 8, true, 4, 8, 58, 165>;    // window sums < 2^16
-using T2 = Tile<104, 4, 5, 4, false, 4, 4, 26, 211>;  // 32-bit prefixes
+using T1 = Tile<96, 4, 7, 8, true, 4, 8, 58, 158>;    // window sums < 2^16
+using T2 = Tile<104, 4, 5, 4, false, 4, 4, 26, 200>;  // 32-bit prefixes
 using T3 = Tile<104, 4, 7, 4, false, 4, 4, 58, 236>;  // 32-bit prefixes
-using T4 = Tile<64, 4, 5, 16, true, 4, 16, 46, 93>;  // narrow frames, window sums < 2^16
-using T5 = Tile<100, 4, 5, 8, true, 4, 8, 28, 141>;   // window sums < 2^16
+using T4 = Tile<64, 4, 5, 16, true, 4, 16, 46, 108>; // narrow frames, window sums < 2^16
+using T5 = Tile<100, 4, 5, 8, true, 4, 8, 28, 136>;   // window sums < 2^16
 // slabs of 8 disparities: two threads per column, 32-bit prefixes (the
 // batch autotuner's deeper slab)
 using T6 = Tile<48, 8, 5, 4, false, 4, 4, 52, 259>;
 // wide horizontal windows (Table I: W_x up to 141 per side), wx <= 174,
 // 32-bit prefixes; 64 columns leave room for 8 producer warps and row slots
-using T7 = Tile<64, 4, 13, 8, false, 4, 8, 174, 180>;
+using T7 = Tile<64, 4, 13, 8, false, 4, 8, 174, 205>;
 // wx up to 66 (Table I's W_x = 61) with 32-bit prefixes: 7 prefix entries
 // per producer lane leave room for 8 producer warps and row slots
 using T8 = Tile<88, 4, 7, 8, false, 4, 8, 66, 170>;
@@ -700,8 +704,8 @@ using T8 = Tile<88, 4, 7, 8, false, 4, 8, 66, 170>;
 // their total need not (W_x 41 and 61 at cost scale 512): packed prefixes after
 // all, with one more load per window. Faster than four 32-bit prefixes a row
 // (1436 x 992, W_x 41: 134 -> 94 us, W_x 61: 160 -> 140 us).
-using T3S = Tile<96, 4, 7, 8, true, 4, 8, 58, 166, true>;
-using T8S = Tile<88, 4, 7, 12, true, 4, 12, 66, 140, true>;
+using T3S = Tile<96, 4, 7, 8, true, 4, 8, 58, 160, true>;
+using T8S = Tile<88, 4, 7, 12, true, 4, 12, 66, 148, true>;
 bool split_fits(const CostAggArgs &a)
 {
     return (uint64_t)std::max(a.wx + 1, T3S::KE) * a.P < 65536u;
