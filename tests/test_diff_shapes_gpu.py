@@ -114,3 +114,15 @@ def test_workspace_holds_only_planes_in_use():
                               torch.from_numpy(ru).cuda(), D, TAU, st)
     assert e.value.code == _lib.STEREO_ENOMEM
     st.close()
+
+
+# windows of one row or one column, spans past 32 cells, arms at every cap, wide
+# windows, one pair more than a support launch takes, segments' and bands' edges,
+# more disparities than columns
+@pytest.mark.parametrize("B,W,H,D,wx,wy", [(1, 70, 40, 12, 0, 0), (2, 65, 33, 9, 21, 0), (1, 40, 70, 9, 0, 31),
+                                           (1, 120, 90, 20, 21, 31), (1, 90, 70, 8, 5, 5), (1, 300, 80, 12, 141, 31),
+                                           (1, 261, 67, 17, 61, 15), (33, 31, 9, 5, 21, 31), (1, 1100, 9, 24, 21, 31),
+                                           (1, 505, 6, 8, 21, 31), (1, 506, 6, 9, 21, 31), (1, 3, 40, 16, 21, 31),
+                                           (1, 20, 12, 64, 21, 31)])
+def test_windows_segments_and_batches(B, W, H, D, wx, wy):
+    _check(B, W, H, D, wx, wy)
