@@ -520,11 +520,12 @@ __host__ __device__ __forceinline__ int hgrad_segments(int X) { return (X + kHSe
 // Blocks of a pair and chunk, each with one partial.
 int hgrad_blocks(int X, int Y) { return hgrad_segments(X) * ((Y + kHRows - 1) / kHRows); }
 
-// s += v with the rounding error carried along in c (Kahan).
+// s += v with the rounding error carried along in c (Kahan). A sum that overflows
+// stays infinite: its error, inf - inf at the next term, would make it NaN.
 __device__ __forceinline__ void kahan(float &s, float &c, float v)
 {
-    const float y = __fsub_rn(v, c), t = __fadd_rn(s, y);
-    c = __fsub_rn(__fsub_rn(t, s), y);
+    const float y = __fsub_rn(v, c), t = __fadd_rn(s, y), e = __fsub_rn(__fsub_rn(t, s), y);
+    c = fabsf(e) < INFINITY ? e : 0.f;
     s = t;
 }
 __global__ void __launch_bounds__(kHNT) diff_hgrad_kernel(

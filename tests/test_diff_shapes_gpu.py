@@ -126,3 +126,24 @@ def test_workspace_holds_only_planes_in_use():
                                            (1, 20, 12, 64, 21, 31)])
 def test_windows_segments_and_batches(B, W, H, D, wx, wy):
     _check(B, W, H, D, wx, wy)
+
+
+def test_overflowing_parameter_gradient_stays_infinite():
+    # Windows of one pixel, two disparities: the left image is the right one, its
+    # columns take two greys in turn, so only the cells of disparity 1 have a cost and
+    # every pixel's share of d/d w_AD and d/d w_MC is about -1.8e38, of d/d lambda_AD
+    # 1e37: the sums pass the largest float in one direction.
+    from paper_2212_00488_gb300 import Stereo
+    from paper_2212_00488_gb300.diff import soft_argmin_disparity
+    W, H = 400, 4
+    im = np.where(np.arange(W) % 2 == 0, 51, 153).astype(np.uint8)
+    im = np.ascontiguousarray(np.broadcast_to(im[None, None, :, None], (1, H, W, 3)))
+    u = torch.from_numpy(im).cuda()
+    f = u.float() / 255
+    theta = torch.tensor([0.05, 0.0, 0.3, 2.3], device="cuda", requires_grad=True)
+    st = Stereo(0, downscale=0, wx=0, wy=0)
+    dhat = soft_argmin_disparity(f, f.clone(), theta, u, u.clone(), 2, 0.1, st)
+    gt, = torch.autograd.grad(dhat, (theta,), torch.full((1, H, W), 1e38, device="cuda"))
+    st.close()
+    inf = float("inf")
+    assert gt[:3].tolist() == [-inf, -inf, inf]
