@@ -679,17 +679,18 @@ __global__ void __launch_bounds__(T::NT, 1) costagg_batch_kernel(const __grid_co
 
 // Tile shapes (XS x DS, KE, RS, 16-bit prefixes, DPT, producer warps, largest
 // wx, ns per row step). The times are what fits the frames of a sweep that keep
-// every SM busy, relative to tile 0 (at 718 x 496 x 73 alone tile 4 takes 93 where it
-// takes 108 in frames of several waves, and was picked there at a loss of up to 17 %;
-// sweep of 83 frames: picks 1.2 % from the best tile on average before, 0.6 % now).
+// every SM busy, relative to tile 0: at 718 x 496 x 73 alone tile 4 takes 93, in
+// frames of several waves 106, where it was picked at a loss of up to 17 % (sweep of
+// 83 frames: picks 1.2 % from the best tile on average before, 0.6 % now; 210 pairs
+// of 320 to 3840 columns: 1 % less time on average, up to 12 % less and 4 % more).
 // One CTA per SM; the ring of 64 prefix rows per (column, disparity, base)
 // dominates shared memory. Every shape gives the same keys.
 using T0 = Tile<96, 4, 5, 12, true, 4, 12, 26, 121>;  // window sums < 2^16; at 718 columns 8 strips for every slab
 using T1 = Tile<96, 4, 7, 8, true, 4, 8, 58, 158>;    // window sums < 2^16
 using T2 = Tile<104, 4, 5, 4, false, 4, 4, 26, 200>;  // 32-bit prefixes
 using T3 = Tile<104, 4, 7, 4, false, 4, 4, 58, 236>;  // 32-bit prefixes
-using T4 = Tile<64, 4, 5, 16, true, 4, 16, 46, 108>; // narrow frames, window sums < 2^16
-using T5 = Tile<100, 4, 5, 8, true, 4, 8, 28, 136>;   // window sums < 2^16
+using T4 = Tile<64, 4, 5, 16, true, 4, 16, 46, 106>; // narrow frames, window sums < 2^16
+using T5 = Tile<100, 4, 5, 8, true, 4, 8, 28, 141>;   // window sums < 2^16
 // slabs of 8 disparities: two threads per column, 32-bit prefixes (the
 // batch autotuner's deeper slab)
 using T6 = Tile<48, 8, 5, 4, false, 4, 4, 52, 259>;
