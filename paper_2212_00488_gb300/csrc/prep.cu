@@ -6,6 +6,8 @@
 // support pass stages them in shared memory.
 #include "internal.cuh"
 
+#include <type_traits>
+
 namespace stereo {
 namespace {
 
@@ -188,8 +190,8 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__
 
 // Support data: mini-census code and the four cross arms of every pixel.
 //
-// A CTA takes kSX x kSY pixels of one image. Sixteen warps scan: warp w
-// follows direction w / 4 (left, right, up, down) for the row quad w % 4, a
+// A CTA takes kSX x SY pixels of one image, with a warp per row. Each warp
+// follows one direction (left, right, up, down) for one row quad, a
 // lane holding four adjacent pixels as the bytes of one word. A step moves all
 // four to the next pixel of the arm: the shifted word is a funnel shift of two
 // staged words (left, right) or the word of the next row (up, down), |I - c|
@@ -201,24 +203,21 @@ __global__ void __launch_bounds__(kGDT) grey_down_kernel(const __grid_constant__
 // border, so an arm that reaches it would never end there by itself. Bound by the ALU pipe. At 718 x 496 (two
 // images) 34.5 us with one thread following each arm eight pixels at a time
 // and a queue for the arms that go on, 16.5 us now (cold L2, both).
-constexpr int kSX = 128, kSY = 16;           // pixels of a CTA
-constexpr int kSupNT = 512;                  // 4 directions x 4 row quads
-constexpr int kSupWarps = kSupNT / 32;
-constexpr int kSupStage = 5;                 // staged column words per thread and pass
-static_assert(kSupWarps == 4 * (kSY / 4) && kSupWarps == kSY, "a warp per (direction, quad), and per census row");
+constexpr int kSX = 128;                     // columns of a CTA
 constexpr uint32_t kHi = 0x80808080u;
 
 // Words staged beyond each side of a row: a scan of wx steps reads that far,
 // the census reads two pixels.
 __host__ __device__ constexpr int sup_hw(int wx) { return wx > 4 ? (wx + 3) / 4 : 1; }
 __host__ __device__ constexpr int sup_row_words(int wx) { return kSX / 4 + 2 * sup_hw(wx); }
-// Shared memory: staged rows [kSY + 2][row words], staged columns [kSY + 2 wy]
-// [kSX / 4], results [5][kSY][kSX / 4] (four arms, census), all in words.
+// Shared memory: staged rows [SY + 2][row words], staged columns [SY + 2 wy]
+// [kSX / 4], results [5][SY][kSX / 4] (four arms, census), all in words.
+template <int SY>
 __host__ __device__ constexpr int sup_smem(int wx, int wy)
 {
-    return 4 * ((kSY + 2) * sup_row_words(wx) + (kSY + 2 * wy) * (kSX / 4) + 5 * kSY * (kSX / 4));
+    return 4 * ((SY + 2) * sup_row_words(wx) + (SY + 2 * wy) * (kSX / 4) + 5 * SY * (kSX / 4));
 }
-static_assert(sup_smem(kMaxWx, kMaxWy) <= 48 * 1024, "fits the default shared memory of a CTA");
+static_assert(sup_smem<16>(kMaxWx, kMaxWy) <= 48 * 1024, "fits the default shared memory of a CTA");
 
 // Four pixels x .. x + 3 of row `row` (columns clamped to the image; x is a
 // multiple of 4). The pixels come from the aligned words that hold them: a word
@@ -245,31 +244,32 @@ __device__ __forceinline__ uint32_t load_quad(const uint8_t *row, int x, int X)
 
 // Stages the rows of the horizontal scans and the columns of the vertical ones,
 // the loads of one pass (a 21 x 31 window takes one) before its first store.
-template <bool kNarrow>
+template <bool kNarrow, int SY>
 __device__ __forceinline__ void stage(const SupImage &I, uint32_t *rows, uint32_t *cols, int x0, int y0, int hw, int wy)
 {
-    constexpr int P = kSX / 4, B = kSupStage;
+    constexpr int P = kSX / 4, NT = 32 * SY;
+    constexpr int B = (SY + 2 * kMaxWy + SY - 1) / SY;        // column words of a thread, all at once
     const int X = I.X, Y = I.Y, RW = P + 2 * hw, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i0 = threadIdx.x; i0 < (kSY + 2) * RW; i0 += 2 * kSupNT) {
+    for (int i0 = threadIdx.x; i0 < (SY + 2) * RW; i0 += 2 * NT) {
         uint32_t v[2];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const int i = min(i0 + k * kSupNT, (kSY + 2) * RW - 1), r = i / RW;
+            const int i = min(i0 + k * NT, (SY + 2) * RW - 1), r = i / RW;
             v[k] = load_quad<kNarrow>(I.g + (size_t)min(max(y0 - 1 + r, 0), Y - 1) * X, x0 + 4 * (i - r * RW - hw), X);
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if (i0 + k * kSupNT < (kSY + 2) * RW) rows[i0 + k * kSupNT] = v[k];
+            if (i0 + k * NT < (SY + 2) * RW) rows[i0 + k * NT] = v[k];
     }
     if (!I.arm) return;
-    for (int r = warp; r < kSY + 2 * wy; r += B * kSupWarps) {
+    for (int r = warp; r < SY + 2 * wy; r += B * SY) {
         uint32_t v[B];
 #pragma unroll
         for (int k = 0; k < B; ++k)
-            v[k] = load_quad<kNarrow>(I.g + (size_t)min(max(y0 - wy + r + k * kSupWarps, 0), Y - 1) * X, x0 + 4 * lane, X);
+            v[k] = load_quad<kNarrow>(I.g + (size_t)min(max(y0 - wy + r + k * SY, 0), Y - 1) * X, x0 + 4 * lane, X);
 #pragma unroll
         for (int k = 0; k < B; ++k)
-            if (r + k * kSupWarps < kSY + 2 * wy) cols[(r + k * kSupWarps) * P + lane] = v[k];
+            if (r + k * SY < SY + 2 * wy) cols[(r + k * SY) * P + lane] = v[k];
     }
 }
 
@@ -358,8 +358,8 @@ struct SupArgs {
     SupImage im[N];
 };
 
-template <int N, bool kBig, int kPerSM>
-__global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_constant__ SupArgs<N> A)
+template <int N, bool kBig, int SY, int kPerSM>
+__global__ void __launch_bounds__(32 * SY, kPerSM) support_kernel(const __grid_constant__ SupArgs<N> A)
 {
     extern __shared__ __align__(16) uint32_t sup[];
     pdl_trigger();
@@ -368,24 +368,24 @@ __global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_co
     const SupImage I = A.im[im];
     const int X = I.X, Y = I.Y, wx = A.wx, wy = A.wy;
     const int tile = blockIdx.x - A.start[im], tyi = tile / I.nx;
-    const int x0 = (tile - tyi * I.nx) * kSX, y0 = tyi * kSY;
+    const int x0 = (tile - tyi * I.nx) * kSX, y0 = tyi * SY;
     const int hw = sup_hw(wx), RW = kSX / 4 + 2 * hw;
     constexpr int P = kSX / 4;
-    uint32_t *rows = sup;                                  // [kSY + 2][RW], from row y0 - 1, word -hw
-    uint32_t *cols = rows + (kSY + 2) * RW;                // [kSY + 2 wy][P], from row y0 - wy
-    uint32_t *res = cols + (kSY + 2 * wy) * P;             // [5][kSY][P]
+    uint32_t *rows = sup;                                  // [SY + 2][RW], from row y0 - 1, word -hw
+    uint32_t *cols = rows + (SY + 2) * RW;                 // [SY + 2 wy][P], from row y0 - wy
+    uint32_t *res = cols + (SY + 2 * wy) * P;              // [5][SY][P]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     pdl_wait();                                            // the grey image of the previous kernel
     if ((blockIdx.x | threadIdx.x) == 0) *A.err = 0u;
 
     if (X >= 4)
-        stage<false>(I, rows, cols, x0, y0, hw, wy);
+        stage<false, SY>(I, rows, cols, x0, y0, hw, wy);
     else
-        stage<true>(I, rows, cols, x0, y0, hw, wy);
+        stage<true, SY>(I, rows, cols, x0, y0, hw, wy);
     __syncthreads();
 
     if (I.arm) {
-        const int dir = warp >> 2, q = warp & 3;
+        const int dir = warp / (SY / 4), q = warp % (SY / 4);
         const uint32_t bm = (uint32_t)(A.tc - (kBig ? 128 : 0)) * 0x01010101u;
         uint32_t n[4];
         const uint32_t *rw = rows + (1 + 4 * q) * RW + hw + lane, *cl = cols + (wy + 4 * q) * P + lane;
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_co
         else
             scan_y<kBig, 1>(cl, min(wy, Y - 1 - (y0 + 4 * q)), bm, n);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) res[(dir * kSY + 4 * q + j) * P + lane] = n[j];
+        for (int j = 0; j < 4; ++j) res[(dir * SY + 4 * q + j) * P + lane] = n[j];
     }
     {
         // census of row `warp` (Fig. 3 is missing: six neighbours in rows y-1..y+1,
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_co
             const uint32_t t = (nb[k] | kHi) - cl;         // bit 7: the low seven bits are not darker
             code |= (((~nb[k] & c) | (~(nb[k] ^ c) & ~t)) & kHi) >> (7 - k);
         }
-        res[(4 * kSY + warp) * P + lane] = code;
+        res[(4 * SY + warp) * P + lane] = code;
     }
     __syncthreads();
 
@@ -428,12 +428,12 @@ __global__ void __launch_bounds__(kSupNT, kPerSM) support_kernel(const __grid_co
         const int y = y0 + 4 * q + j;
         if (y >= Y) break;
         const size_t i = (size_t)y * X + x;
-        I.pix[i] = (uint32_t)gb[4 * j * RW] | (uint32_t)rb[(4 * kSY + j) * kSX] << 8;
+        I.pix[i] = (uint32_t)gb[4 * j * RW] | (uint32_t)rb[(4 * SY + j) * kSX] << 8;
         if (I.key) I.key[i] = 0xFFFFFFFFu;         // WTA key preset: the fused kernel takes atomic minima
         if (!I.arm) continue;
         // the scans run over clamped pixels: arms end at the image border
-        const int l = min((int)rb[j * kSX], x), r = min((int)rb[(kSY + j) * kSX], X - 1 - x);
-        const int u = min((int)rb[(2 * kSY + j) * kSX], y), d = min((int)rb[(3 * kSY + j) * kSX], Y - 1 - y);
+        const int l = min((int)rb[j * kSX], x), r = min((int)rb[(SY + j) * kSX], X - 1 - x);
+        const int u = min((int)rb[(2 * SY + j) * kSX], y), d = min((int)rb[(3 * SY + j) * kSX], Y - 1 - y);
         I.arm[i] = pack_arm(l, r, u, d);
         if (!I.armc) continue;
         uint16_t *ac = reinterpret_cast<uint16_t *>(I.armc);
@@ -526,32 +526,43 @@ template <int N>
 cudaError_t support_run(const SupImage *im, int n, int wx, int wy, int tc, uint32_t *err, cudaStream_t s)
 {
     SupArgs<N> A;
+    const auto lay = [&](int sy) {                        // CTAs of sy rows
+        A.start[0] = 0;
+        for (int i = 0; i < n; ++i) A.start[i + 1] = A.start[i] + A.im[i].nx * ((im[i].Y + sy - 1) / sy);
+        return A.start[n];
+    };
     A.n = n;
     A.wx = wx;
     A.wy = wy;
     A.tc = tc;
     A.err = err;
-    A.start[0] = 0;
     for (int i = 0; i < n; ++i) {
         A.im[i] = im[i];
         A.im[i].nx = (im[i].X + kSX - 1) / kSX;
-        A.start[i + 1] = A.start[i] + A.im[i].nx * ((im[i].Y + kSY - 1) / kSY);
     }
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const auto go = [&](auto kernel) {
-        return launch_dependent(kernel, dim3(A.start[n]), dim3(kSupNT), sup_smem(wx, wy), s, A);
+    const auto go = [&](auto rows, auto kernel, auto big) {
+        constexpr int SY = decltype(rows)::value;
+        return launch_dependent(tc < 128 ? kernel : big, dim3(A.start[n]), dim3(32 * SY), sup_smem<SY>(wx, wy), s, A);
     };
+    using std::integral_constant;
+    // Frames whose CTAs of eight rows all get an SM of their own: an SM then issues
+    // half the scan steps (W_x 21, flat blocks: 64 x 48 6.3 -> 5.1 us, 381 x 195 9.6 ->
+    // 6.9; W_x 141: 114 x 44 17.0 -> 14.6 us). The halo of two such CTAs costs more than that
+    // where an SM has several (718 x 496: 21.5 against 16.9 us).
+    if (lay(8) <= sms)
+        return go(integral_constant<int, 8>{}, support_kernel<N, false, 8, 2>, support_kernel<N, true, 8, 2>);
     // Images whose CTAs all run at once with two on an SM take the form with 64
     // registers, which has more scan steps' loads in flight; more CTAs take
-    // three on an SM (40 registers). 360 x 248: 15.9 -> 11.4 us, 640 x 480 (300
-    // CTAs): 14.7 -> 11.4 us; at 372 and 544 CTAs there is nothing to choose,
-    // from 2040 (3840 x 2160, halved) three are the faster, 66.7 against 64.4 us.
-    if (A.start[n] <= 2 * sms)
-        return tc < 128 ? go(support_kernel<N, false, 2>) : go(support_kernel<N, true, 2>);
-    return tc < 128 ? go(support_kernel<N, false, 3>) : go(support_kernel<N, true, 3>);
+    // three on an SM (40 registers). Flat blocks, W_x 21, 64 against 40 registers, launches in a
+    // row: 512 x 384 (192 CTAs) 12.0 and 14.4 us, 640 x 400 (250) 11.7 and 16.1; past two on an SM
+    // 718 x 496 (372) 16.7 and 16.6, 960 x 540 (544) 21.0 and 20.6, 1920 x 1080 (2040) 67.5 and 65.2.
+    if (lay(16) <= 2 * sms)
+        return go(integral_constant<int, 16>{}, support_kernel<N, false, 16, 2>, support_kernel<N, true, 16, 2>);
+    return go(integral_constant<int, 16>{}, support_kernel<N, false, 16, 3>, support_kernel<N, true, 16, 3>);
 }
 
 }  // namespace
