@@ -42,3 +42,11 @@ def test_codes_and_arms_at_tile_edges(W, H, tc, wx, wy):
         assert np.array_equal(got["census_" + side].cpu().numpy(), oracle.census(g))
         assert np.array_equal(got["arms_" + side].cpu().numpy().view(np.uint32).astype(np.int64), want)
     st.close()
+
+
+# either side of the line up to which CTAs of eight rows each have an SM (150 and
+# 156 of them on 152 SMs), and with fewer than four columns
+@pytest.mark.parametrize("W,H", [(300, 200), (300, 208), (2, 30)])
+@pytest.mark.parametrize("tc,wx,wy", [(13, 21, 31), (200, 141, 31), (40, 61, 7), (13, 0, 0)])
+def test_rows_of_a_cta(W, H, tc, wx, wy):
+    test_codes_and_arms_at_tile_edges(W, H, tc, wx, wy)
