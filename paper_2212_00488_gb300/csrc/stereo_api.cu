@@ -120,6 +120,7 @@ int fail(stereo_ctx *c, int code, const char *fmt, ...)
 
 int cuda_fail(stereo_ctx *c, cudaError_t e, const char *what)
 {
+    cudaGetLastError();   // the runtime's copy of the error, which a later launch would take for its own
     return fail(c, STEREO_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

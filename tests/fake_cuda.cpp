@@ -1,6 +1,8 @@
 // A CUDA runtime and the library's launchers for tests of csrc/stereo_api.cu on
 // the CPU: every call succeeds and does nothing but write its line to a log, except
-// the one launch that fake_fail_at() names, which returns an error.
+// the one launch that fake_fail_at() names and the capture queries while
+// fake_fail_query() is on. As in the runtime, an error also stays until
+// cudaGetLastError() takes it, and a launch without a status of its own asks that.
 #include "internal.cuh"
 
 #include <cstdlib>
@@ -13,6 +15,8 @@ using namespace stereo;
 namespace {
 std::string g_log;
 int g_launch = 0, g_fail = -1, g_nodes = 0;
+bool g_fail_query = false;
+cudaError_t g_last = cudaSuccess;
 uintptr_t g_next = 0x1000;
 bool g_capturing = false;
 
@@ -29,7 +33,8 @@ cudaError_t launch(const char *name, cudaStream_t s, int *launches = nullptr)
     say(std::string("launch ") + name + " " + hex(s));
     ++g_nodes;
     if (launches) ++*launches;
-    return g_launch++ == g_fail ? cudaErrorLaunchFailure : cudaSuccess;
+    if (g_launch++ == g_fail) return g_last = cudaErrorLaunchFailure;
+    return cudaSuccess;
 }
 }  // namespace
 
@@ -39,8 +44,11 @@ STEREO_TEST_API void fake_reset()
     g_log.clear();
     g_launch = 0;
     g_fail = -1;
+    g_fail_query = false;
+    g_last = cudaSuccess;
 }
 STEREO_TEST_API void fake_fail_at(int launch) { g_fail = launch; }
+STEREO_TEST_API void fake_fail_query(int on) { g_fail_query = on != 0; }
 STEREO_TEST_API const char *fake_log() { return g_log.c_str(); }
 }
 
@@ -54,7 +62,8 @@ bool costagg_fits(const CostAggArgs &a, int tile) { return tile != 0 || (uint64_
 int costagg_pick(const CostAggArgs &a, int) { return costagg_fits(a, 0) ? 0 : 1; }
 cudaError_t launch_grey(const uint8_t *, const uint8_t *, uint8_t *, uint8_t *, int, int, cudaStream_t s)
 {
-    return launch("grey", s);
+    launch("grey", s);
+    return cudaGetLastError();
 }
 cudaError_t launch_grey_down(const GreyJob *jobs, int n, cudaStream_t s, int *launches)
 {
@@ -107,7 +116,12 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int)
     p->multiProcessorCount = 152;
     return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError()
+{
+    const cudaError_t e = g_last;
+    g_last = cudaSuccess;
+    return e;
+}
 const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "a call failed"; }
 cudaError_t cudaMalloc(void **p, size_t n) { return *p = malloc(n), cudaSuccess; }
 cudaError_t cudaFree(void *p) { return free(p), cudaSuccess; }
@@ -136,6 +150,7 @@ cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.f, cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *c)
 {
+    if (g_fail_query) return g_last = cudaErrorStreamCaptureImplicit;
     return *c = cudaStreamCaptureStatusNone, cudaSuccess;
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode)

@@ -148,3 +148,22 @@ def test_a_frame_takes_the_planes_it_uses(fake, downscale):
     # words, the fused kernel's arm words (whole row quads), keys; medians and filled map
     planes = [W * H] * downscale + [n] * 2 + [4 * n] * 6 + [4 * X * ((Y + p.wy + 3) // 4 * 4)] * 2 + [n, 4 * n]
     assert _lib.stereo_job_bytes(p, W, H, 64) == sum((b + 255) // 256 * 256 for b in planes) + 256
+
+
+@pytest.mark.parametrize("what", ["query", "launch"])
+def test_a_call_after_one_that_failed_is_not_refused_for_it(fake, what):
+    # the runtime keeps a failed call's error until it is asked for, and the grey
+    # conversion's launch reports what it is then told
+    ctx = _context(downscale=0)
+    _lib.stereo_set_tile(ctx, 1)
+    fake.fake_reset()
+    if what == "query":
+        fake.fake_fail_query(1)
+    else:
+        fake.fake_fail_at(3)
+    with pytest.raises(_lib.StereoError):
+        _lib.stereo_compute_batch(ctx, _jobs([80, 80]), CALLER)
+    fake.fake_fail_query(0)
+    fake.fake_fail_at(-1)
+    _lib.stereo_compute(ctx, 1, 1, 80, 60, 16, 1, 0, 0, 0, CALLER)
+    _lib.stereo_destroy(ctx)
