@@ -20,7 +20,7 @@
 //    in the rest. The sweep starts wy rows above the band and ends wy below.
 //
 // What bounds it: the instructions of the few warps an SM has room for beside
-// the ring (issue slots 60-70 % used, shared-memory pipe 75 %). 718 x 496 x 73:
+// the ring (issue slots 55 % used, shared-memory pipe 83 %). 718 x 496 x 73:
 // 68.6 us, from 80.8 us with 100 columns, 7 + 12 warps and halfword loads for
 // the right base. The steps: packed prefixes in plain 32-bit adds with one
 // 8-byte load per window end for both bases (one path for all warps), the ring
@@ -622,8 +622,8 @@ __host__ __device__ __forceinline__ int slab_strips(const CostAggArgs &a, int sl
 
 // CTA t of a frame: the first a.head tiles (strip, slab) of a.tiles are swept from
 // the first row to the last, the others in row bands of a.band rows: all of them
-// in the first band, then in the next. (The count comes with the arguments: adding
-// it up over the slabs cost a CTA 1.2 us at 26 slabs.)
+// in the first band, then in the next. (The count comes with the arguments: with
+// every CTA adding it up over the slabs, 3283 x 16 x 104, W_x 61, took 69.8 us for 65.6.)
 template <class T>
 __device__ __forceinline__ void run_tile(const CostAggArgs &a, int t, unsigned char *smem, bool reuse)
 {
