@@ -517,8 +517,15 @@ static_assert(kHRows * kHSeg / kHB * kDC / 2 == kHNT, "one (row, band, disparity
 constexpr int kHPitch = kHNT + 1;
 constexpr int kHSmem = (kHB + 1) * kHPitch * (int)sizeof(float2);
 __host__ __device__ __forceinline__ int hgrad_segments(int X) { return (X + kHSeg - kDC) / (kHSeg - kDC + 1); }
-// Blocks of a pair and chunk, each with one partial.
-int hgrad_blocks(int X, int Y) { return hgrad_segments(X) * ((Y + kHRows - 1) / kHRows); }
+// Rows of a block, a multiple of kHRows, and blocks of a pair and chunk. Each has one
+// partial of 16 bytes: images of a few columns with many chunks take more rows a
+// block, so that the partials stay below about 50 bytes a pixel.
+int hgrad_rows(int X, int nchunks) { return kHRows * std::max(1, nchunks * hgrad_segments(X) / (4 * X)); }
+int hgrad_blocks(int X, int Y, int nchunks)
+{
+    const int rows = hgrad_rows(X, nchunks);
+    return hgrad_segments(X) * ((Y + rows - 1) / rows);
+}
 
 // s += v with the rounding error carried along in c (Kahan). A sum that overflows
 // stays infinite: its error, inf - inf at the next term, would make it NaN.
@@ -562,8 +569,8 @@ __global__ void __launch_bounds__(kHNT) diff_hgrad_kernel(
     const float ea1 = expf(-inv_lad);
     const int kn = min(kDC, D - d0);
     float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f, e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
-    // (`rows` is kHRows: the loop runs once, but written without it the kernel gets
-    // other code, 80 registers for 92, and a step at 4 x 718 x 496 takes 4.77 ms, not 4.61)
+    // (once for kHRows; without the loop the kernel gets other code, 80 registers for
+    // 92, and a step at 4 x 718 x 496 takes 4.77 ms, not 4.61)
     const int y_end = min(((int)blockIdx.y + 1) * rows, Y);
     for (int y = blockIdx.y * rows; y < y_end; y += kHRows) {
         const int nr = min(kHRows, y_end - y);
@@ -824,7 +831,7 @@ size_t diff_layout(char *base, int X, int Y, int B, int D, DiffWs *w)
     t.s0 = (float *)take(nb * kDC * n * 4);                  // slabs: x sums, their gradient, its vertical adjoint
     t.s1 = (float *)take(nb * kDC * n * 4);
     t.s2 = (float *)take(nb * kDC * n * 4);
-    t.part = (float *)take(nb * nchunks * hgrad_blocks(X, Y) * 16);   // parameter-gradient partials
+    t.part = (float *)take(nb * nchunks * hgrad_blocks(X, Y, (int)nchunks) * 16);   // parameter-gradient partials
     t.seg = (double *)take(kRedBlocks * 4 * sizeof(double)); // their segment sums
     if (w) *w = t;
     return off;
@@ -852,8 +859,8 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
     diff_layout((char *)a.ws, X, Y, B, a.D, &w);
     const int nblk = (n + kDiffNT - 1) / kDiffNT;
     const int nchunks = (a.D + kDC - 1) / kDC;
-    const int nseg = hgrad_segments(X), yblocks = (Y + kHRows - 1) / kHRows;
-    const size_t part_chunk = (size_t)hgrad_blocks(X, Y) * 4, part_pair = part_chunk * nchunks;
+    const int nseg = hgrad_segments(X), rows = hgrad_rows(X, nchunks), yblocks = (Y + rows - 1) / rows;
+    const size_t part_chunk = (size_t)hgrad_blocks(X, Y, nchunks) * 4, part_pair = part_chunk * nchunks;
     const float inv_tau = 1.f / a.tau;
     const dim3 tiles((X + kTileX - 1) / kTileX, (Y + kTileY - 1) / kTileY, B);
     static_assert(kTileX == 32 && kTileX * kTileY == kDiffNT, "one thread per pixel of a tile, a warp per row");
@@ -898,7 +905,7 @@ cudaError_t diff_run(const DiffArgs &a, cudaStream_t s)
                 cudaSuccess)
             break;
         e = launch_dependent(diff_hgrad_kernel, dim3(nseg, yblocks, B), dim3(kHNT), 0, s, w.s2,
-                             w.arml, w.gl, w.gr, w.pixl, w.pixr, a.theta, X, Y, a.D, d0, a.wx, kHRows, c == 0, w.accl,
+                             w.arml, w.gl, w.gr, w.pixl, w.pixr, a.theta, X, Y, a.D, d0, a.wx, rows, c == 0, w.accl,
                              w.accr, w.part + c * part_chunk, part_pair);
     }
     if (e != cudaSuccess) return e;

@@ -84,20 +84,20 @@ def _check(B, W, H, D, wx, wy, seed=0):
 
 # few pixels, many chunks of disparities: more partials of the parameter gradients than pixels
 @pytest.mark.parametrize("B,W,H,D,wy", [(64, 1, 1, 256, 31), (4, 1, 1, 256, 31), (16, 1, 12, 256, 31),
-                                        (3, 4, 4, 256, 0), (8, 3, 8, 256, 0)])
+                                        (3, 4, 4, 256, 0), (8, 3, 8, 256, 0), (2, 2, 70, 256, 31)])
 def test_images_of_a_few_pixels(B, W, H, D, wy):
     _check(B, W, H, D, 21, wy)
 
 
-def test_workspace_holds_only_planes_in_use():
-    # 142 bytes a pixel and pair, and the partials (16 bytes for two rows of a
-    # segment and chunk): a context capped at 150 bytes a pixel runs the step
+# 142 bytes a pixel and pair, and the partials (16 bytes for two rows of a segment
+# and chunk, fewer in narrow images): capped contexts run the step
+@pytest.mark.parametrize("B,W,H,D,cap_per_pixel", [(2, 300, 200, 24, 150), (1, 2, 4000, 256, 200)])
+def test_workspace_holds_only_planes_in_use(B, W, H, D, cap_per_pixel):
     from paper_2212_00488_gb300 import Stereo, _lib
     from paper_2212_00488_gb300.diff import soft_argmin_disparity
-    B, W, H, D = 2, 300, 200, 24
     lu, ru, go = _grey_images(B, W, H, 3)
     res = []
-    for cap in (0, 150 * B * W * H):
+    for cap in (0, cap_per_pixel * B * W * H):
         st = Stereo(0, downscale=0, mem_cap_bytes=cap)
         l, r = (torch.from_numpy(a.astype(np.float32) / 255).cuda().requires_grad_(True) for a in (lu, ru))
         theta = torch.tensor(THETA, device="cuda", requires_grad=True)
